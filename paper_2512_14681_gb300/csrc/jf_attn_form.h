@@ -1,11 +1,11 @@
 // Launch form of the split-KV attention (host side; no CUDA types, so that the rule compiles and is
 // tested on the host alone).
 //
-// A unit (chain, KV head, tile of 128 query rows) runs on 8 CTAs, one key lane each. The clustered
-// form makes them an 8-CTA cluster and folds the lane states in parallel after a cluster barrier,
-// but only `max_clusters` such clusters are resident at once (15 on a GB300: 120 of 152 SMs). The
-// unclustered form can use every SM, and the last lane of a unit folds all its rows. Both fold in
-// lane order with the same arithmetic, so the choice affects time only.
+// A unit (chain, KV head, tile of 128 query rows) has 8 key lanes, spread over 8, 4, 2 or 1 CTAs (one
+// cluster; one CTA per SM). max_clusters[i] clusters of 2^i CTAs are resident at once (152, 76, 36, 15
+// on a GB300). Wide clusters shorten a unit, narrow ones fit more units at once and fold less through
+// memory. Every form computes the same lane states and folds them in the same order, so the choice
+// affects time only.
 #pragma once
 
 namespace jf {
@@ -20,13 +20,26 @@ inline int attn_units_estimate(int M, int chains, int units_bound, int Hkv, int 
   return est < units_bound ? (int)est : units_bound;
 }
 
-// true: the clustered form, which is taken unless the unclustered one needs fewer waves of units
-// (ties go to the clustered form, whose parallel fold is faster).
+// true: clusters of `max_clusters` at once need no more waves of units than `lanes` independent places
+// per unit on `num_sms` of them do.
 inline bool attn_use_clusters(int units, int lanes, int max_clusters, int num_sms) {
   const int mc = max_clusters > 0 ? max_clusters : 1;
   const int waves_clustered = (units + mc - 1) / mc;
   const int waves_unclustered = (int)(((long long)units * lanes + num_sms - 1) / num_sms);
   return waves_clustered <= waves_unclustered;
+}
+
+// CTAs per unit: the widest clusters that need no more waves than the next narrower ones. Past one wave
+// of single CTAs, pairs when their waves (half as long, plus about an eighth of a single CTA's for the
+// prologue and the fold) are the shorter. One 7B layer (4 KV heads, 7 query heads each), us with
+// 8 / 4 / 2 / 1 CTAs per unit: 8 units at P = 4096 116 / 122 / 134 / 146; 16 units 131 / 128 / 140 / 150;
+// 36 units at 2048 168 / 149 / 158 / 158; 56 units at 4096 220 / 205 / 198 / 204; 112 units 373 / 343 /
+// 331 / 309.
+inline int attn_ctas_per_unit(int units, const int (&max_clusters)[4]) {
+  for (int i = 3; i > 0; --i)
+    if (attn_use_clusters(units, 1, max_clusters[i], max_clusters[i - 1])) return 1 << i;
+  const int w1 = (units + max_clusters[0] - 1) / max_clusters[0], w2 = (units + max_clusters[1] - 1) / max_clusters[1];
+  return w2 * 5 < w1 * 9 ? 2 : 1;
 }
 
 }  // namespace jf

@@ -649,7 +649,8 @@ __global__ void k_commit(const CommitInfo* commit, const uint8_t* k_inf, const u
       continue;
     }
     const int h = v / vec_per_head, w = v % vec_per_head;
-    const size_t dst = ((((size_t)l * n_pages + page) * Hkv + h) * kPage + (p & 15)) * head_bytes + (size_t)w * 16;
+    const size_t in_page = es == 2 ? (size_t)kv_page_offset(p & 15, w) : (size_t)(p & 15) * head_bytes + (size_t)w * 16;
+    const size_t dst = (((size_t)l * n_pages + page) * Hkv + h) * kPage * head_bytes + in_page;
     const size_t src = (size_t)(ci.row0 + j) * row_bytes + (size_t)v * 16;
     *reinterpret_cast<uint4*>(k_pages + dst) = *reinterpret_cast<const uint4*>(ksrc + src);
     *reinterpret_cast<uint4*>(v_pages + dst) = *reinterpret_cast<const uint4*>(vsrc + src);

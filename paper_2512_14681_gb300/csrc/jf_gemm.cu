@@ -380,10 +380,6 @@ JF_DEV Unit unit_of(const GemmParams& p, int u) {
 // ---------------------------------------------------------------------------------------------
 constexpr int TC_THREADS = 192;
 
-JF_DEV void mbar_arrive(uint32_t bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
-}
-
 template <int BN, int EPI>
 __global__ void __launch_bounds__(TC_THREADS, 1)
     k_gemm_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const GemmParams p) {

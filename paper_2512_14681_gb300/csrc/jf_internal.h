@@ -29,12 +29,23 @@ constexpr int kPage = 16;         // tokens per KV page
 constexpr int kTileN = 128;       // weight rows per GEMM tile (tcgen05 M)
 constexpr int kTileK = 64;        // K elements per GEMM pipeline stage
 constexpr int kAttnChunk = 128;   // keys per split-KV chunk, aligned to absolute positions
-constexpr int kAttnQRows = 128;   // (token, head) query rows per attention work unit
+constexpr int kAttnQRows = 128;   // most (token, head) query rows per attention work unit
+// Query rows of a unit's tile with G query heads per KV head: as many whole tokens as fit, so that one
+// TMA box (G heads x tokens) loads them; a group wider than the tile is cut anywhere.
+__host__ __device__ constexpr int attn_tile_rows(int G) { return G <= kAttnQRows ? kAttnQRows / G * G : kAttnQRows; }
 constexpr int kAttnLanes = 8;     // chunk lanes per unit (c mod 8); one CTA of an 8-CTA cluster each
 constexpr int kAttnLaneChunks = 128;  // chunks per lane the kernel can stage page ids for
 constexpr int kAttnMaxCtx = kAttnChunk * kAttnLanes * kAttnLaneChunks;  // 131072 key positions
 constexpr int kAttnXchgFloats = kAttnQRows * 128 + 2 * kAttnQRows;   // one lane state: O (hd 128), m, l
 constexpr int kMaxSeqs = 64;
+
+// A page of one head in a 16-bit K/V pool (head_dim 128) holds its 16 keys x 256 bytes as the image of
+// a tensor-core operand: 8-key groups of 2048 bytes, each two 64-dim halves of 8 rows x 128 bytes with
+// the 128-byte swizzle. A page then is one contiguous copy into shared memory. Byte offset of 16-byte
+// piece c (0..15) of key r (0..15):
+__host__ __device__ constexpr int kv_page_offset(int r, int c) {
+  return (r >> 3) * 2048 + (c >> 3) * 1024 + (r & 7) * 128 + (((c & 7) ^ (r & 7)) << 4);
+}
 constexpr int kMaxChains = 256;
 
 // A chain: in-flight rows row0 .. row0+nrows-1 of sequence `seq` at consecutive positions
@@ -44,7 +55,7 @@ struct Chain {
   int seq, row0, nrows, pos0;
 };
 
-// Attention work unit: (chain, KV head, tile of 128 (token, head) query rows), its chain resolved;
+// Attention work unit: (chain, KV head, tile of (token, head) query rows), its chain resolved;
 // `pad` is nonzero for a unit that exists.
 struct AttnUnit {
   int seq, row0, nrows, pos0, kvh, qt, n_chunks, pad;
@@ -106,7 +117,7 @@ struct AttnParams {
   const void* q;        // [R][Hq][hd]
   const void* k_inf;    // this layer's in-flight K [R][Hkv][hd]
   const void* v_inf;
-  const void* k_pages;  // this layer's K pages [n_pages][Hkv][16][hd]
+  const void* k_pages;  // this layer's K pages [n_pages][Hkv][16][hd] (16-bit pools: kv_page_offset)
   const void* v_pages;
   const int* page_table;  // [max_seqs][pages_per_seq]
   int pages_per_seq;
@@ -120,7 +131,12 @@ struct AttnParams {
   int* err;
   unsigned long long wait_ns;  // limit of each bounded wait
   float* xchg;          // bf16 path: lane states [unit][lane][kAttnXchgFloats]
-  int* unit_ticket;     // bf16 path, unclustered form: lanes finished per unit, zero between launches
+};
+
+// TMA tensors of one layer's queries and in-flight K and V rows (bf16 path), all [row][head][128]: Q in
+// boxes of 64 x G x tokens of a tile, K and V of 64 x 1 x 8 (half of 8 keys of one head).
+struct AttnMaps {
+  CUtensorMap q, k_inf, v_inf;
 };
 
 // Host-side launch helpers of the projection GEMM (jf_gemm.cu) and the TMA descriptor encoder

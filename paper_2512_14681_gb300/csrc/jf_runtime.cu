@@ -28,11 +28,11 @@ cudaError_t launch_rmsnorm(float* x, const float* gain, void* y, bool is_bf16, i
                            const SplitPartials* acc, int row0, cudaStream_t st);
 cudaError_t launch_qkv_finish(const SplitPartials& sp, const void* bias, const int* pos, const float2* rope, void* q,
                               void* k, void* v, int M, int Hq, int Hkv, cudaStream_t st);
-cudaError_t launch_attn_tc(const AttnParams& a, int units_bound, bool clustered, cudaStream_t st);
+cudaError_t launch_attn_tc(const AttnMaps& tm, const AttnParams& a, int units_bound, int n_ctas, cudaStream_t st);
 cudaError_t launch_attn_f32(const AttnParams& a, int n_rows, cudaStream_t st);
 cudaError_t launch_wait_probe(int* err, unsigned long long* waited_ns, unsigned long long limit_ns, cudaStream_t st);
 cudaError_t gemm_prepare();
-cudaError_t attn_prepare(int* max_clusters);
+cudaError_t attn_prepare(int max_clusters[4]);
 }  // namespace jf
 
 using namespace jf;
@@ -84,6 +84,18 @@ bool make_tmap(CUtensorMap* tm, const void* ptr, long long K, long long rows, in
   return r == CUDA_SUCCESS;
 }
 
+// 16-bit rank-3 tensor (dims and box innermost first, strides of the outer dims in bytes), 128-byte
+// swizzle.
+bool make_tmap_3d(CUtensorMap* tm, const void* ptr, const cuuint64_t (&dims)[3], const cuuint64_t (&strides)[2],
+                  const cuuint32_t (&box)[3]) {
+  if (!get_encode()) return false;
+  cuuint32_t es[3] = {1, 1, 1};
+  CUresult r = g_encode(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(ptr), dims, strides, box, es,
+                        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  return r == CUDA_SUCCESS;
+}
+
 // ------------------------------------------------------------------------------------------
 // Arena plan: offsets of every device buffer, shared by jf_arena_bytes and jf_create.
 // ------------------------------------------------------------------------------------------
@@ -112,7 +124,7 @@ struct Offsets {
   std::vector<size_t> w_qkv, w_o, w_gu, w_d, g_attn, g_mlp, b_qkv;
   size_t k_pages, v_pages, page_table, seq_len, commit;
   size_t k_inf, v_inf, x, h, q, att, act;
-  size_t tok, pos, gpred, top2, chains, n_chains, attn_xchg, attn_ticket;
+  size_t tok, pos, gpred, top2, chains, n_chains, attn_xchg;
   size_t gemm_ws, gemm_counter, am_v1, am_i1, am_v2, am_counter;
   size_t logits, err, traj_count;
   size_t gen_state, gen_out, gen_truth, gen_log, gen_q0, gen_plast, gen_prompt, gen_seqp, res, step_blocks, step_res,
@@ -168,7 +180,7 @@ jf_status make_dims(const jf_model_config* m, const jf_runtime_config* rt, Dims*
   }
   D->max_chains = rt->max_segments > 0 ? rt->max_segments : std::min(kMaxChains, D->S * 5 + 1);
   if (D->bf16) {
-    D->max_units = D->Hkv * (cdiv((long long)D->R * D->G, kAttnQRows) + D->max_chains);
+    D->max_units = D->Hkv * (cdiv((long long)D->R * D->G, attn_tile_rows(D->G)) + D->max_chains);
   } else {
     D->max_units = 1;
   }
@@ -230,7 +242,6 @@ Offsets plan_offsets(const Dims& D) {
   o.n_chains = p.take(16);
   // attention lane states: [unit][lane][128 x 128 O, 128 m, 128 l] fp32 (bf16 path)
   o.attn_xchg = p.take(D.bf16 ? (size_t)D.max_units * kAttnLanes * kAttnXchgFloats * 4 : 16, 1024);
-  o.attn_ticket = p.take((size_t)D.max_units * 4);
   o.gemm_ws_bytes = gemm_ws_floats(D) * 4;
   o.gemm_ws = p.take(std::max<size_t>(o.gemm_ws_bytes, 16), 1024);
   const int max_mt = cdiv(D.R, 16) + 1;
@@ -263,6 +274,7 @@ struct LayerW {
   void* b_qkv;  // [nq + 2 nkv] in the model dtype, or null
   float *g_attn, *g_mlp;
   CUtensorMap tm_qkv, tm_o, tm_gu, tm_dn;
+  AttnMaps tm_attn;
 };
 
 struct GraphRec {
@@ -309,8 +321,7 @@ struct jf_ctx {
   Chain* chains;
   int* n_chains;
   float* attn_xchg;
-  int* attn_ticket;
-  int attn_max_clusters = 0;  // 8-CTA clusters of the attention resident at once
+  int attn_max_clusters[4] = {};  // clusters of 1, 2, 4, 8 CTAs of the attention resident at once
   int chains_bound = 1;  // most chains the next forward can have (sizes the attention launch)
   float* gemm_ws;
   int* gemm_counter;
@@ -542,15 +553,13 @@ cudaError_t enqueue_forward(jf_ctx* c, int M, LmMode lm) {
     a.err = c->err;
     a.wait_ns = c->wait_ns;
     a.xchg = c->attn_xchg;
-    a.unit_ticket = c->attn_ticket;
     prof_begin(c, PC_ATTN);
     if (D.bf16) {
       // units of this forward are bounded by its rows: every chain adds at most one partial tile
-      const int units_bound = std::min(D.max_units, D.Hkv * (cdiv((long long)M * D.G, kAttnQRows) + c->chains_bound));
-      // clustered unless the unclustered form needs fewer waves of units (jf_attn_form.h)
-      const int units_est = attn_units_estimate(M, c->chains_bound, units_bound, D.Hkv, D.G, kAttnQRows);
-      e = launch_attn_tc(a, units_bound, attn_use_clusters(units_est, kAttnLanes, c->attn_max_clusters, c->num_sms),
-                         c->st);
+      const int tile = attn_tile_rows(D.G);
+      const int units_bound = std::min(D.max_units, D.Hkv * (cdiv((long long)M * D.G, tile) + c->chains_bound));
+      const int units_est = attn_units_estimate(M, c->chains_bound, units_bound, D.Hkv, D.G, tile);
+      e = launch_attn_tc(w.tm_attn, a, units_bound, attn_ctas_per_unit(units_est, c->attn_max_clusters), c->st);
       prof_end(c);
     } else {
       e = launch_attn_f32(a, M, c->st);
@@ -1034,9 +1043,26 @@ jf_status jf_create(const jf_model_config* model, const jf_runtime_config* rt, j
   c->commit = at<CommitInfo>(c, O.commit);
   c->k_inf = at<void>(c, O.k_inf);
   c->v_inf = at<void>(c, O.v_inf);
+  c->q = at<void>(c, O.q);
+  if (D.bf16) {
+    const size_t inf_layer = (size_t)D.R * D.nkv * D.es;
+    const cuuint64_t row = (cuuint64_t)D.hd * 2;
+    const cuuint64_t rows = (cuuint64_t)D.R, hd = (cuuint64_t)D.hd;
+    const cuuint64_t dims[3] = {hd, (cuuint64_t)D.Hkv, rows}, strides[2] = {row, row * D.Hkv};
+    const cuuint64_t q_dims[3] = {hd, (cuuint64_t)D.Hq, rows}, q_strides[2] = {row, row * D.Hq};
+    const cuuint32_t box[3] = {64, 1, 8};
+    const cuuint32_t heads = std::min(D.G, kAttnQRows);  // (a wider group does not use the tensor)
+    const cuuint32_t q_box[3] = {64, heads, (cuuint32_t)kAttnQRows / heads};
+    for (int l = 0; l < D.L; ++l) {
+      AttnMaps& m = c->layers[l].tm_attn;
+      if (!make_tmap_3d(&m.q, c->q, q_dims, q_strides, q_box) ||
+          !make_tmap_3d(&m.k_inf, reinterpret_cast<char*>(c->k_inf) + l * inf_layer, dims, strides, box) ||
+          !make_tmap_3d(&m.v_inf, reinterpret_cast<char*>(c->v_inf) + l * inf_layer, dims, strides, box))
+        return abandon(JF_ECUDA);
+    }
+  }
   c->x = at<float>(c, O.x);
   c->h = at<void>(c, O.h);
-  c->q = at<void>(c, O.q);
   c->att = at<void>(c, O.att);
   c->act = at<void>(c, O.act);
   c->tok = at<int>(c, O.tok);
@@ -1045,7 +1071,6 @@ jf_status jf_create(const jf_model_config* model, const jf_runtime_config* rt, j
   c->top2 = at<float>(c, O.top2);
   c->chains = at<Chain>(c, O.chains);
   c->attn_xchg = at<float>(c, O.attn_xchg);
-  c->attn_ticket = at<int>(c, O.attn_ticket);
   c->n_chains = at<int>(c, O.n_chains);
   c->gemm_ws = at<float>(c, O.gemm_ws);
   c->gemm_counter = at<int>(c, O.gemm_counter);
@@ -1083,7 +1108,6 @@ jf_status jf_create(const jf_model_config* model, const jf_runtime_config* rt, j
   zero(O.gemm_counter, (O.am_v1 - O.gemm_counter));
   zero(O.am_counter, (size_t)(cdiv(D.R, 16) + 1) * 4);
   zero(O.err, 16);
-  zero(O.attn_ticket, (size_t)D.max_units * 4);
   zero(O.n_chains, 16);
   zero(O.x, (size_t)D.R * D.d * 4);
   zero(O.h, (size_t)D.R * D.d * D.es);
@@ -1092,7 +1116,7 @@ jf_status jf_create(const jf_model_config* model, const jf_runtime_config* rt, j
   if (e == cudaSuccess) e = cudaMemsetAsync(c->page_table, 0xff, (size_t)D.S * D.pps * 4, c->st);
   if (e == cudaSuccess) e = launch_rope_table(c->rope, D.max_ctx + 1, D.hd / 2, c->mc.rope_theta, c->st);
   if (e == cudaSuccess) e = gemm_prepare();
-  if (e == cudaSuccess) e = attn_prepare(&c->attn_max_clusters);
+  if (e == cudaSuccess) e = attn_prepare(c->attn_max_clusters);
   if (e == cudaSuccess) e = cudaStreamSynchronize(c->st);
   if (e != cudaSuccess) return abandon(JF_ECUDA);
   *out = c;
