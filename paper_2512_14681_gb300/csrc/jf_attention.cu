@@ -666,13 +666,20 @@ __global__ void __launch_bounds__(ATT_THREADS, 1)
   JF_TL_EXIT(TL_ATTN);
 }
 
-// fp32 path: one warp per (row, query head); keys in absolute order, 32 at a time.
+// fp32 path: one warp per (row, query head); keys in absolute order, 32 at a time. Latency bounds it
+// (small models, short contexts): a lane has its whole key row in flight at once (four partial dot
+// products), and the value rows are loaded eight at a time before their sums.
+template <int HDT>
 __global__ void __launch_bounds__(128) k_attn_f32(const AttnParams a, int n_rows) {
-  const int warp_global = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  constexpr int NV = HDT / 32;  // dims per lane of the output
+  __shared__ float4 s_q[4][HDT / 4];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int job = blockIdx.x * 4 + warp;
+  pdl_launch_dependents();
   pdl_wait();
-  const int r = warp_global / a.Hq, h = warp_global % a.Hq;
+  const int r = job / a.Hq, h = job % a.Hq;
   if (r >= n_rows) return;
-  const int hd = a.hd, G = a.Hq / a.Hkv, kvh = h / G;
+  const int kvh = h / (a.Hq / a.Hkv);
   const int n_ch = *a.n_chains_dev;
   int ci = 0;
   for (; ci < n_ch; ++ci) {
@@ -682,60 +689,79 @@ __global__ void __launch_bounds__(128) k_attn_f32(const AttnParams a, int n_rows
   if (ci == n_ch) return;
   const Chain ch = a.chains[ci];
   const int pos = ch.pos0 + (r - ch.row0);
-  const float* q = reinterpret_cast<const float*>(a.q) + ((size_t)r * a.Hq + h) * hd;
+  const float4* q = reinterpret_cast<const float4*>(reinterpret_cast<const float*>(a.q) + ((size_t)r * a.Hq + h) * HDT);
+  if (lane < HDT / 4) s_q[warp][lane] = q[lane];
+  __syncwarp();
   const float* Kp = reinterpret_cast<const float*>(a.k_pages);
   const float* Vp = reinterpret_cast<const float*>(a.v_pages);
   const float* Ki = reinterpret_cast<const float*>(a.k_inf);
   const float* Vi = reinterpret_cast<const float*>(a.v_inf);
   const float scale = a.scale_log2;
-  float m = -INFINITY, l = 0.f, o0 = 0.f, o1 = 0.f;
+  float m = -INFINITY, l = 0.f, o[NV];
+#pragma unroll
+  for (int i = 0; i < NV; ++i) o[i] = 0.f;
   for (int kb = 0; kb <= pos; kb += 32) {
     const int kp = kb + lane;
     float s = -INFINITY;
-    const float* kr = nullptr;
+    unsigned long long v_row = 0;  // this lane's key's value row
     if (kp <= pos) {
+      size_t off;
       if (kp < ch.pos0) {
         const int page = a.page_table[(size_t)ch.seq * a.pages_per_seq + (kp >> 4)];
-        const size_t off = (((size_t)page * a.Hkv + kvh) * kPage + (kp & 15)) * hd;
-        kr = Kp + off;
+        off = (((size_t)page * a.Hkv + kvh) * kPage + (kp & 15)) * HDT;
       } else {
-        const size_t off = ((size_t)(ch.row0 + kp - ch.pos0) * a.Hkv + kvh) * hd;
-        kr = Ki + off;
+        off = ((size_t)(ch.row0 + kp - ch.pos0) * a.Hkv + kvh) * HDT;
       }
-      float dot = 0.f;
-      for (int i = 0; i < hd; ++i) dot = fmaf(q[i], kr[i], dot);
-      s = dot * scale;
+      const float4* kr = reinterpret_cast<const float4*>((kp < ch.pos0 ? Kp : Ki) + off);
+      v_row = reinterpret_cast<unsigned long long>((kp < ch.pos0 ? Vp : Vi) + off);
+      float d[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+      for (int i0 = 0; i0 < HDT / 4; i0 += 16) {
+        float4 kv[16];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) kv[i] = kr[i0 + i];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+          const float4 x = s_q[warp][i0 + i];
+          d[0] = fmaf(x.x, kv[i].x, d[0]);
+          d[1] = fmaf(x.y, kv[i].y, d[1]);
+          d[2] = fmaf(x.z, kv[i].z, d[2]);
+          d[3] = fmaf(x.w, kv[i].w, d[3]);
+        }
+      }
+      s = ((d[0] + d[1]) + (d[2] + d[3])) * scale;
     }
     float mx = s;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    for (int sh = 16; sh > 0; sh >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, sh));
     const float mn = fmaxf(m, mx);
     const float al = (m == -INFINITY) ? 0.f : exp2f(m - mn);
     const float p = (s == -INFINITY) ? 0.f : exp2f(s - mn);
-    float ps = warp_sum(p);
-    l = l * al + ps;
-    o0 *= al;
-    o1 *= al;
-    for (int j = 0; j < 32; ++j) {
-      const float pj = __shfl_sync(0xffffffffu, p, j);
-      const int kpj = kb + j;
-      if (kpj > pos) break;
-      const float* vrow;
-      if (kpj < ch.pos0) {
-        const int page = a.page_table[(size_t)ch.seq * a.pages_per_seq + (kpj >> 4)];
-        vrow = Vp + (((size_t)page * a.Hkv + kvh) * kPage + (kpj & 15)) * hd;
-      } else {
-        vrow = Vi + ((size_t)(ch.row0 + kpj - ch.pos0) * a.Hkv + kvh) * hd;
+    l = l * al + warp_sum(p);
+#pragma unroll
+    for (int i = 0; i < NV; ++i) o[i] *= al;
+    for (int j0 = 0; j0 < 32 && kb + j0 <= pos; j0 += 8) {
+      float v[8][NV], pj[8];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const float* vr = reinterpret_cast<const float*>(__shfl_sync(0xffffffffu, v_row, j0 + j));
+        pj[j] = __shfl_sync(0xffffffffu, p, j0 + j);
+#pragma unroll
+        for (int i = 0; i < NV; ++i) v[j][i] = (kb + j0 + j <= pos) ? vr[lane + 32 * i] : 0.f;
       }
-      o0 = fmaf(pj, vrow[lane], o0);
-      if (lane + 32 < hd) o1 = fmaf(pj, vrow[lane + 32], o1);
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        if (kb + j0 + j > pos) break;
+#pragma unroll
+        for (int i = 0; i < NV; ++i) o[i] = fmaf(pj[j], v[j][i], o[i]);
+      }
     }
     m = mn;
   }
-  float* out = reinterpret_cast<float*>(a.out) + ((size_t)r * a.Hq + h) * hd;
+  float* out = reinterpret_cast<float*>(a.out) + ((size_t)r * a.Hq + h) * HDT;
   const float il = l > 0.f ? 1.f / l : 0.f;
-  out[lane] = o0 * il;
-  if (lane + 32 < hd) out[lane + 32] = o1 * il;
+#pragma unroll
+  for (int i = 0; i < NV; ++i) out[lane + 32 * i] = o[i] * il;
 }
 
 }  // namespace
@@ -800,7 +826,7 @@ cudaError_t launch_attn_f32(const AttnParams& a, int n_rows, cudaStream_t st) {
   at[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k_attn_f32, a, n_rows);
+  return cudaLaunchKernelEx(&cfg, a.hd == 64 ? k_attn_f32<64> : k_attn_f32<128>, a, n_rows);
 }
 
 }  // namespace jf

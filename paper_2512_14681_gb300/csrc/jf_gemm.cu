@@ -7,7 +7,7 @@
 // tiles by TMA (128-byte swizzle) through a 4-12 stage mbarrier ring that never drains between
 // units; an MMA warp accumulates into one of two TMEM accumulators; four epilogue warps drain
 // the other accumulator (fused epilogue, split-K reduction) while the next unit streams in.
-// fp32 path (small fp32 models): a SIMT mainloop with the same tile shape and epilogues.
+// fp32 path (small fp32 models): a SIMT mainloop over 128-feature tiles with the same epilogues.
 //
 // Split-K is deterministic: partial tiles go to a workspace and the last CTA of a tile (atomic
 // ticket, no waiting) adds them in split order. Every output element's reduction order is fixed
@@ -260,14 +260,14 @@ JF_DEV void argmax_finish(const GemmEpi& e, int m0, int BN, int n_slots, int tid
 
 template <typename T, int BN, int EPI, typename Get>
 JF_DEV void finish_tile_epi(const GemmParams& p, Get get, float* xs, int* sflag, int n_tile, int split, int m_tile,
-                            int tid, int n0, int m0, int tile_lin, int nchunks);
+                            int tid, int slot, int n_slots, int n0, int m0, int tile_lin, int nchunks);
 
 // Shared tail of both mainloops, run by the 128 epilogue threads (tid 0..127): the partial tile
 // for EPI_PARTIAL; otherwise ticketing for split-K and argmax, then the epilogue. get(c0, v) fills
-// this thread's 16 accumulator values of columns c0..c0+15.
+// this thread's 16 accumulator values of columns c0..c0+15. slot of n_slots: this CTA's argmax slots.
 template <typename T, int BN, int EPI, typename Get>
 JF_DEV void finish_tile(const GemmParams& p, Get get, float* xs, int* sflag, int n_tile, int split, int m_tile,
-                        int tid) {
+                        int tid, int slot, int n_slots) {
   const int n0 = n_tile * kTileN, m0 = m_tile * BN;
   const int tile_lin = n_tile * p.m_tiles + m_tile;
   int ncols = p.M - m0;
@@ -282,18 +282,19 @@ JF_DEV void finish_tile(const GemmParams& p, Get get, float* xs, int* sflag, int
       for (int j = 0; j < 16; ++j) mine[(c * 16 + j) * kTileN + tid] = v[j];
     }
   } else {
-    finish_tile_epi<T, BN, EPI>(p, get, xs, sflag, n_tile, split, m_tile, tid, n0, m0, tile_lin, nchunks);
+    finish_tile_epi<T, BN, EPI>(p, get, xs, sflag, n_tile, split, m_tile, tid, slot, n_slots, n0, m0, tile_lin,
+                                  nchunks);
   }
 }
 
 template <typename T, int BN, int EPI, typename Get>
 JF_DEV void finish_tile_epi(const GemmParams& p, Get get, float* xs, int* sflag, int n_tile, int split, int m_tile,
-                            int tid, int n0, int m0, int tile_lin, int nchunks) {
+                            int tid, int slot, int n_slots, int n0, int m0, int tile_lin, int nchunks) {
   if (p.k_splits == 1) {
     for (int c = 0; c < nchunks; ++c) {
       float v[16];
       get(c * 16, v);
-      epilogue_chunk<T, EPI>(p.epi, v, tid, n0, m0, c * 16, xs, n_tile, blockIdx.x, gridDim.x);
+      epilogue_chunk<T, EPI>(p.epi, v, tid, n0, m0, c * 16, xs, n_tile, slot, n_slots);
     }
   } else {
     float* mine = p.ws + ((size_t)tile_lin * p.k_splits + split) * (size_t)BN * kTileN;
@@ -334,7 +335,7 @@ JF_DEV void finish_tile_epi(const GemmParams& p, Get get, float* xs, int* sflag,
           for (int j = 0; j < 16; ++j) v[j] += part[s][j];
         }
       }
-      epilogue_chunk<T, EPI>(p.epi, v, tid, n0, m0, c * 16, xs, n_tile, blockIdx.x, gridDim.x);
+      epilogue_chunk<T, EPI>(p.epi, v, tid, n0, m0, c * 16, xs, n_tile, slot, n_slots);
     }
     if (tid == 0) p.tile_counter[tile_lin] = 0;
   }
@@ -350,7 +351,7 @@ JF_DEV void finish_tile_epi(const GemmParams& p, Get get, float* xs, int* sflag,
     epi_sync();
     if (last) {
       __threadfence();
-      argmax_finish(p.epi, m0, BN, gridDim.x, tid);
+      argmax_finish(p.epi, m0, BN, n_slots, tid);
       if (tid == 0) p.epi.am_counter[m_tile] = 0;
     }
   }
@@ -542,7 +543,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
       tc_fence_after();
       const uint32_t dacc = tmem + (uint32_t)(acc * Cfg::ACC_COLS) + lane_base;
       auto get = [&](int c0, float (&v)[16]) { tmem_ld16(dacc + (uint32_t)c0, v); };
-      finish_tile<bf16, BN, EPI>(p, get, xs, sflag, w.n_tile, w.split, w.m_tile, tid);
+      finish_tile<bf16, BN, EPI>(p, get, xs, sflag, w.n_tile, w.split, w.m_tile, tid, blockIdx.x, gridDim.x);
       tc_fence_before();
       epi_sync();
       if (tid == 0) mbar_arrive(tempty0 + 8 * acc);
@@ -555,59 +556,124 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
 }
 
 // ---------------------------------------------------------------------------------------------
-// fp32 SIMT kernel: thread `row` accumulates Y[m0 .. m0+31, n0 + row] over K in fp32, in
-// increasing k, with the token tile staged in shared memory.
+// fp32 SIMT kernel: a cluster of n_splits CTAs per tile of 128 features x BN tokens, each CTA on its
+// share of K. Weight and token tiles of 32 k stream through shared memory by cp.async (four stages);
+// thread (row, h) sums Y[m0 .. m0+BN-1, n0 + row] over the k of half h of every tile; the halves, then
+// the CTAs of the cluster in rank order (read from their shared memory), are added in a fixed order that
+// depends on N and K alone. These models' matrices are small (a 256 x 1024 one is two feature tiles), so
+// latency bounds the kernel: it is spread over 8-152 SMs instead of one CTA per tile whose threads each
+// walked a weight row (a jf_op_gemm call of 4096 x 1024, 40 rows: 158 -> 41 us, most of which is now the
+// call itself; the tiny fp32 decoder's generation, with the fp32 attention: 35.6 -> 6.9 ms).
 // ---------------------------------------------------------------------------------------------
-constexpr int F32_BN = 32;
 constexpr int F32_BK = 32;
+constexpr int F32_STAGES = 4;
+constexpr int F32_PITCH = F32_BK + 4;  // floats per tile row: 16-byte aligned, conflict-free 16-byte reads
+constexpr int F32_THREADS = 256;
+constexpr int f32_stage_floats(int bn) { return (kTileN + bn) * F32_PITCH; }
+constexpr int f32_smem(int bn) { return F32_STAGES * f32_stage_floats(bn) * 4; }
 
-template <int EPI>
-__global__ void __launch_bounds__(128) k_gemm_f32(const float* __restrict__ W, const float* __restrict__ X,
-                                                  const GemmParams p) {
-  __shared__ float xt[F32_BN][F32_BK + 1];
+// Four consecutive floats of a row (k .. k+3, zeros past K) into shared memory: one 16-byte copy when
+// every row is 16-byte aligned, otherwise four 4-byte ones.
+JF_DEV void f32_copy4(uint32_t dst, const float* row, int k, int K, bool ok, bool vec) {
+  const int left = ok ? K - k : 0;
+  if (vec) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(row + (left > 0 ? k : 0)),
+                 "r"(left > 0 ? 16 : 0)
+                 : "memory");
+  } else {
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst + 4 * i), "l"(row + (left > i ? k + i : 0)),
+                   "r"(left > i ? 4 : 0)
+                   : "memory");
+  }
+}
+
+JF_DEV float ld_cluster_f32(const float* p, uint32_t rank) {  // *p of the cluster's CTA `rank`
+  uint32_t addr;
+  float v;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(addr) : "r"(smem_u32(p)), "r"(rank));
+  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
+  return v;
+}
+
+template <int BN, int EPI>
+__global__ void __launch_bounds__(F32_THREADS) k_gemm_f32(const float* __restrict__ W, const float* __restrict__ X,
+                                                          const GemmParams p, int n_splits, bool vec) {
+  extern __shared__ __align__(16) float tiles[];  // F32_STAGES x {W [128][PITCH], X [BN][PITCH]}
+  __shared__ float part[BN * kTileN];
   __shared__ float xs[16 * 128];
   __shared__ int sflag;
-  const int tid = threadIdx.x;
-  const int n0 = blockIdx.x * kTileN, m0 = blockIdx.z * F32_BN;
-  const int n = n0 + tid;
-  pdl_wait();
-  float acc[F32_BN];
-#pragma unroll
-  for (int j = 0; j < F32_BN; ++j) acc[j] = 0.0f;
-  for (int k0 = 0; k0 < p.K; k0 += F32_BK) {
-    for (int i = tid; i < F32_BN * F32_BK; i += 128) {
-      const int r = i / F32_BK, c = i % F32_BK;
-      const int m = m0 + r, k = k0 + c;
-      xt[r][c] = (m < p.M && k < p.K) ? X[(size_t)m * p.K + k] : 0.0f;
-    }
-    __syncthreads();
-    if (n < p.N) {
-      const float* wr = W + (size_t)n * p.K + k0;
-      const int kmax = (p.K - k0) < F32_BK ? (p.K - k0) : F32_BK;
-      for (int c = 0; c < kmax; ++c) {
-        const float w = wr[c];
-#pragma unroll
-        for (int j = 0; j < F32_BN; ++j) acc[j] = fmaf(w, xt[j][c], acc[j]);
-      }
-    }
-    __syncthreads();
-  }
+  const int tid = threadIdx.x, row = tid & 127, half = tid >> 7;
+  const int n_tile = blockIdx.x / n_splits, split = blockIdx.x % n_splits;
+  const int n0 = n_tile * kTileN, m0 = blockIdx.z * BN;
+  const int kb0 = (int)((long long)p.kb_total * split / n_splits), kb1 = (int)((long long)p.kb_total * (split + 1) / n_splits);
   pdl_launch_dependents();
-  auto get = [&](int c0, float (&v)[16]) {
-#pragma unroll
-    for (int j = 0; j < 16; ++j) v[j] = 0.0f;
-#pragma unroll
-    for (int cc = 0; cc < F32_BN; cc += 16)
-      if (cc == c0) {
-#pragma unroll
-        for (int j = 0; j < 16; ++j) v[j] = acc[cc + j];
-      }
+  pdl_wait();
+  auto load = [&](int kb) {
+    const uint32_t base = smem_u32(tiles + ((kb - kb0) % F32_STAGES) * f32_stage_floats(BN));
+    for (int i = tid; i < (kTileN + BN) * (F32_BK / 4); i += F32_THREADS) {
+      const int r = i / (F32_BK / 4), c = (i % (F32_BK / 4)) * 4;
+      const bool w = r < kTileN;
+      const int g = w ? n0 + r : m0 + r - kTileN;
+      const bool ok = g < (w ? p.N : p.M);
+      f32_copy4(base + (uint32_t)(r * F32_PITCH + c) * 4, (w ? W : X) + (ok ? (size_t)g * p.K : 0), kb * F32_BK + c, p.K, ok,
+                vec);
+    }
   };
-  if constexpr (EPI == EPI_ARGMAX) {
-    argmax_init_slots(p.epi, m0, m0 + F32_BN, blockIdx.x, gridDim.x, tid, 128);
-    __syncthreads();
+  for (int s = 0; s < F32_STAGES - 1; ++s) {
+    if (kb0 + s < kb1) load(kb0 + s);
+    asm volatile("cp.async.commit_group;" ::: "memory");
   }
-  finish_tile<float, F32_BN, EPI>(p, get, xs, &sflag, blockIdx.x, 0, blockIdx.z, tid);
+  float acc[BN];
+#pragma unroll
+  for (int j = 0; j < BN; ++j) acc[j] = 0.0f;
+  for (int kb = kb0; kb < kb1; ++kb) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(F32_STAGES - 2) : "memory");
+    __syncthreads();  // this tile has landed; the one before it has been read by everyone
+    if (kb + F32_STAGES - 1 < kb1) load(kb + F32_STAGES - 1);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    const float* wt = tiles + ((kb - kb0) % F32_STAGES) * f32_stage_floats(BN) + half * (F32_BK / 2);
+    const float* xt = wt + kTileN * F32_PITCH;
+#pragma unroll
+    for (int k = 0; k < F32_BK / 2; k += 4) {
+      const float4 w = *reinterpret_cast<const float4*>(wt + row * F32_PITCH + k);
+#pragma unroll
+      for (int j = 0; j < BN; ++j) {
+        const float4 x = *reinterpret_cast<const float4*>(xt + j * F32_PITCH + k);
+        acc[j] = fmaf(w.x, x.x, acc[j]);
+        acc[j] = fmaf(w.y, x.y, acc[j]);
+        acc[j] = fmaf(w.z, x.z, acc[j]);
+        acc[j] = fmaf(w.w, x.w, acc[j]);
+      }
+    }
+  }
+  if (half == 1) {
+#pragma unroll
+    for (int j = 0; j < BN; ++j) part[j * kTileN + row] = acc[j];
+  }
+  __syncthreads();
+  if (half == 0) {
+#pragma unroll
+    for (int j = 0; j < BN; ++j) part[j * kTileN + row] += acc[j];
+  }
+  if (n_splits > 1) cluster_sync();  // every CTA's partial tile is visible to rank 0
+  if (split == 0 && half == 0) {
+    auto get = [&](int c0, float (&v)[16]) {
+#pragma unroll
+      for (int j = 0; j < 16; ++j) v[j] = part[(c0 + j) * kTileN + row];
+      for (int r = 1; r < n_splits; ++r) {
+#pragma unroll
+        for (int j = 0; j < 16; ++j) v[j] += ld_cluster_f32(part + (c0 + j) * kTileN + row, (uint32_t)r);
+      }
+    };
+    if constexpr (EPI == EPI_ARGMAX) {
+      argmax_init_slots(p.epi, m0, m0 + BN, n_tile, p.n_tiles, tid, 128);
+      epi_sync();
+    }
+    finish_tile<float, BN, EPI>(p, get, xs, &sflag, n_tile, 0, blockIdx.z, tid, n_tile, p.n_tiles);
+  }
+  if (n_splits > 1) cluster_sync();  // the other CTAs keep their partial tiles until rank 0 has read them
 }
 
 template <int BN, int EPI>
@@ -658,9 +724,22 @@ cudaError_t prep_tc() {
 JF_TL_SETTER(tl_set_gemm)
 #endif
 
-// Opt the tcgen05 kernels into their dynamic shared-memory sizes on the current device.
+template <int BN>
+static cudaError_t prep_f32() {
+  cudaError_t e;
+  const int sm = f32_smem(BN);
+  if ((e = cudaFuncSetAttribute(k_gemm_f32<BN, EPI_STORE>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm))) return e;
+  if ((e = cudaFuncSetAttribute(k_gemm_f32<BN, EPI_RESID>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm))) return e;
+  if ((e = cudaFuncSetAttribute(k_gemm_f32<BN, EPI_QKV>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm))) return e;
+  if ((e = cudaFuncSetAttribute(k_gemm_f32<BN, EPI_SWIGLU>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm))) return e;
+  return cudaFuncSetAttribute(k_gemm_f32<BN, EPI_ARGMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+}
+
+// Opt the kernels into their dynamic shared-memory sizes on the current device.
 static cudaError_t gemm_prepare_current() {
   cudaError_t e;
+  if ((e = prep_f32<16>()) != cudaSuccess) return e;
+  if ((e = prep_f32<32>()) != cudaSuccess) return e;
   if ((e = prep_tc<32>()) != cudaSuccess) return e;
   if ((e = prep_tc<64>()) != cudaSuccess) return e;
   if ((e = prep_tc<128>()) != cudaSuccess) return e;
@@ -718,24 +797,53 @@ cudaError_t launch_gemm_bf16(const CUtensorMap& tmA, const CUtensorMap& tmB, con
   }
 }
 
-cudaError_t launch_gemm_f32(const float* W, const float* X, const GemmParams& p, cudaStream_t st) {
+// CTAs per tile of the fp32 kernel (from N and K alone, so that a row's sums do not depend on the rows in
+// flight): a power of two up to 8, at least 64 k each, about one CTA per SM of a 152-SM GPU at the most.
+static int f32_splits(int n_tiles, int K) {
+  int s = 1;
+  while (s < 8 && 2 * s * 64 <= K && 2 * s * n_tiles <= 152) s *= 2;
+  return s;
+}
+
+template <int BN, int EPI>
+static cudaError_t launch_f32_epi(const float* W, const float* X, GemmParams p, cudaStream_t st) {
+  p.m_tiles = (p.M + BN - 1) / BN;
+  p.kb_total = (p.K + F32_BK - 1) / F32_BK;
+  const int splits = f32_splits(p.n_tiles, p.K);
+  const bool vec = p.K % 4 == 0 && ((reinterpret_cast<uintptr_t>(W) | reinterpret_cast<uintptr_t>(X)) & 15) == 0;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(p.n_tiles, 1, p.m_tiles);
-  cfg.blockDim = dim3(128);
+  cfg.gridDim = dim3(p.n_tiles * splits, 1, p.m_tiles);
+  cfg.blockDim = dim3(F32_THREADS);
+  cfg.dynamicSmemBytes = f32_smem(BN);
   cfg.stream = st;
-  cudaLaunchAttribute at[1];
+  cudaLaunchAttribute at[2];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[0].val.programmaticStreamSerializationAllowed = 1;
+  at[1].id = cudaLaunchAttributeClusterDimension;
+  at[1].val.clusterDim.x = splits;
+  at[1].val.clusterDim.y = 1;
+  at[1].val.clusterDim.z = 1;
   cfg.attrs = at;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = splits > 1 ? 2 : 1;
+  return cudaLaunchKernelEx(&cfg, k_gemm_f32<BN, EPI>, W, X, p, splits, vec);
+}
+
+template <int BN>
+static cudaError_t launch_f32(const float* W, const float* X, const GemmParams& p, cudaStream_t st) {
   switch (p.epi.kind) {
-    case EPI_STORE: return cudaLaunchKernelEx(&cfg, k_gemm_f32<EPI_STORE>, W, X, p);
-    case EPI_RESID: return cudaLaunchKernelEx(&cfg, k_gemm_f32<EPI_RESID>, W, X, p);
-    case EPI_QKV: return cudaLaunchKernelEx(&cfg, k_gemm_f32<EPI_QKV>, W, X, p);
-    case EPI_SWIGLU: return cudaLaunchKernelEx(&cfg, k_gemm_f32<EPI_SWIGLU>, W, X, p);
-    case EPI_ARGMAX: return cudaLaunchKernelEx(&cfg, k_gemm_f32<EPI_ARGMAX>, W, X, p);
+    case EPI_STORE: return launch_f32_epi<BN, EPI_STORE>(W, X, p, st);
+    case EPI_RESID: return launch_f32_epi<BN, EPI_RESID>(W, X, p, st);
+    case EPI_QKV: return launch_f32_epi<BN, EPI_QKV>(W, X, p, st);
+    case EPI_SWIGLU: return launch_f32_epi<BN, EPI_SWIGLU>(W, X, p, st);
+    case EPI_ARGMAX: return launch_f32_epi<BN, EPI_ARGMAX>(W, X, p, st);
     default: return cudaErrorInvalidValue;
   }
+}
+
+cudaError_t launch_gemm_f32(const float* W, const float* X, const GemmParams& p, cudaStream_t st) {
+  // 32-token tiles once they fill the GPU (half the weight reads), 16-token ones below that
+  const long long ctas32 = (long long)p.n_tiles * f32_splits(p.n_tiles, p.K) * ((p.M + 31) / 32);
+  return ctas32 >= 304 ? launch_f32<32>(W, X, p, st) : launch_f32<16>(W, X, p, st);
 }
 
 }  // namespace jf

@@ -494,7 +494,6 @@ cudaError_t gemm(jf_ctx* c, const CUtensorMap& tmA, const void* W, const void* X
     if (!make_tmap(&tmB, X, K, M, bn)) return cudaErrorInvalidValue;
     e = launch_gemm_bf16(tmA, tmB, p, bn, c->st);
   } else {
-    p.m_tiles = cdiv(M, 32);
     p.k_splits = 1;
     e = launch_gemm_f32(reinterpret_cast<const float*>(W), reinterpret_cast<const float*>(X), p, c->st);
   }
@@ -1632,6 +1631,7 @@ jf_status jf_op_gemm(int dtype, const void* W, const void* X, float* Y, int N, i
     if (!make_tmap(&tA, W, K, N, kTileN) || !make_tmap(&tB, X, K, M, bn)) return JF_ECUDA;
     e = launch_gemm_bf16(tA, tB, p, bn, st);
   } else {
+    if (gemm_prepare() != cudaSuccess) return JF_ECUDA;
     e = launch_gemm_f32(reinterpret_cast<const float*>(W), reinterpret_cast<const float*>(X), p, st);
   }
   return e == cudaSuccess ? JF_OK : JF_ECUDA;
