@@ -108,7 +108,8 @@ cudaError_t launch_traj_noisy(const int* traj, int n_rec, int R, int seq, const 
                               int n_blocks, int* noisy, int* point, cudaStream_t st);
 cudaError_t launch_step_accept(const StepBlocks* sb, const int* tok, const int* gpred, int* committed,
                                CommitInfo* commit, StepResult* res, int* err, cudaStream_t st);
-cudaError_t launch_commit(const CommitInfo* commit, int n_seqs, int L, const void* k_inf, const void* v_inf,
+// rows: rows in flight of the forward, an upper bound of what one sequence commits
+cudaError_t launch_commit(const CommitInfo* commit, int n_seqs, int rows, int L, const void* k_inf, const void* v_inf,
                           void* k_pages, void* v_pages, const int* page_table, int pages_per_seq, int n_pages,
                           int max_rows, int Hkv, int hd, int elem_bytes, int* seq_len, int* err, cudaStream_t st);
 

@@ -637,7 +637,7 @@ jf_status prefill_impl(jf_ctx* c, int seq, const int32_t* host_prompt, const int
     CK(enqueue_forward(c, m, last_chunk ? LM_LAST : LM_NONE));
     CommitInfo ci{0, m, P};
     CK(cudaMemcpyAsync(c->commit + seq, &ci, sizeof(ci), cudaMemcpyHostToDevice, c->st));
-    CK(launch_commit(c->commit + seq, 1, D.L, c->k_inf, c->v_inf, c->k_pages, c->v_pages,
+    CK(launch_commit(c->commit + seq, 1, m, D.L, c->k_inf, c->v_inf, c->k_pages, c->v_pages,
                      c->page_table + (size_t)seq * D.pps, D.pps, D.n_pages, D.R, D.Hkv, D.hd, D.es, c->seq_len + seq,
                      c->err, c->st));
     c->launches += 1;
@@ -667,7 +667,7 @@ cudaError_t enqueue_iteration(jf_ctx* c, const GenCfg& g, int M, int n_seqs) {
   prof_end(c);
   if (e != cudaSuccess) return e;
   prof_begin(c, PC_OTHER);
-  e = launch_commit(c->commit, n_seqs, D.L, c->k_inf, c->v_inf, c->k_pages, c->v_pages, c->page_table, D.pps,
+  e = launch_commit(c->commit, n_seqs, M, D.L, c->k_inf, c->v_inf, c->k_pages, c->v_pages, c->page_table, D.pps,
                     D.n_pages, D.R, D.Hkv, D.hd, D.es, c->seq_len, c->err, c->st);
   prof_end(c);
   if (e != cudaSuccess) return e;
@@ -1440,7 +1440,7 @@ jf_status jf_jacobi_step(jf_ctx* c, int seq, int n_blocks, const jf_block* block
   c->chains_bound = nch;
   CK(enqueue_forward(c, total, LM_ARGMAX));
   CK(launch_step_accept(c->sb_dev, c->tok, c->gpred, c->committed_dev, c->commit, c->sres_dev, c->err, c->st));
-  CK(launch_commit(c->commit + seq, 1, D.L, c->k_inf, c->v_inf, c->k_pages, c->v_pages,
+  CK(launch_commit(c->commit + seq, 1, total, D.L, c->k_inf, c->v_inf, c->k_pages, c->v_pages,
                    c->page_table + (size_t)seq * D.pps, D.pps, D.n_pages, D.R, D.Hkv, D.hd, D.es, c->seq_len + seq,
                    c->err, c->st));
   StepResult r;
