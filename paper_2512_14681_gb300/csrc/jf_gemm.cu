@@ -24,9 +24,12 @@ constexpr int A_STAGE_BYTES = kTileN * kTileK * 2;  // 16 KB of weights per stag
 constexpr int EPI_STAGE_BYTES = 16 * kTileN * 4;   // epilogue exchange buffer [16][128] fp32
 constexpr int SMEM_LIMIT = 232448;                  // 227 KB per CTA
 
-template <int BN>
+// PAIR: two CTAs (a cluster) share a tile of 256 weight rows; each stages its 128 rows of A and half of
+// the tile's tokens.
+template <int BN, bool PAIR>
 struct TcCfg {
-  static constexpr int B_STAGE_BYTES = BN * kTileK * 2;
+  static constexpr int B_ROWS = PAIR ? BN / 2 : BN;
+  static constexpr int B_STAGE_BYTES = B_ROWS * kTileK * 2;
   static constexpr int STAGE_BYTES = A_STAGE_BYTES + B_STAGE_BYTES;
   static constexpr int S0 = (SMEM_LIMIT - 1024 - EPI_STAGE_BYTES - 512) / STAGE_BYTES;
   static constexpr int STAGES = S0 < 2 ? 2 : (S0 > 12 ? 12 : S0);
@@ -359,7 +362,7 @@ JF_DEV void finish_tile_epi(const GemmParams& p, Get get, float* xs, int* sflag,
 
 // Work unit u of the persistent schedule: split = u % k_splits; the k_splits units of a tile are
 // consecutive (their partials meet soon), and so are the m tiles of a weight tile (its second
-// read hits L2).
+// read hits L2). n_tile counts pairs of tiles when two CTAs share one.
 struct Unit {
   int n_tile, m_tile, split, kb0, kb1;
 };
@@ -377,15 +380,23 @@ JF_DEV Unit unit_of(const GemmParams& p, int u) {
 // ---------------------------------------------------------------------------------------------
 // bf16 tcgen05 persistent kernel, 192 threads: warps 0-3 epilogue (warp w reads TMEM lanes
 // 32w .. 32w+31), warp 4 lane 0 = TMA producer (warp 4 also owns the TMEM allocation),
-// warp 5 lane 0 = MMA issuer.
+// warp 5 = MMA issuer.
+//
+// PAIR (256-token tiles, i.e. more than 160 rows): two CTAs on neighbouring SMs take a tile of 256
+// weight rows together (cta_group::2). Each loads its own 128 weight rows and half of the tokens (32 KB
+// a 64-k stage instead of 48), rank 0 issues the MMAs of both, and each drains its own 128 rows. With
+// one CTA per tile the operands, not the tensor cores, bounded it: 48 KB a 512-cycle stage is more than
+// an SM draws from L2, and only four such stages fit. gate/up (37888 x 3584) at 512 rows: 110.6 ->
+// 104.9 us a call (1.33 PFLOP/s); prefill of 4,000 tokens through one 7B layer 2.39 -> 2.29 ms.
 // ---------------------------------------------------------------------------------------------
 constexpr int TC_THREADS = 192;
 
-template <int BN, int EPI>
+template <int BN, int EPI, bool PAIR>
 __global__ void __launch_bounds__(TC_THREADS, 1)
     k_gemm_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const GemmParams p) {
-  using Cfg = TcCfg<BN>;
+  using Cfg = TcCfg<BN, PAIR>;
   constexpr int S = Cfg::STAGES;
+  constexpr int kCtas = PAIR ? 2 : 1;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = align1024(smem_raw);
   uint8_t* sA = smem;
@@ -398,7 +409,11 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const uint32_t full0 = smem_u32(bars), empty0 = smem_u32(bars + S);
   const uint32_t tfull0 = smem_u32(bars + 2 * S), tempty0 = smem_u32(bars + 2 * S + 2);
-  const int total_units = p.n_tiles * p.m_tiles * p.k_splits;
+  const int rank = PAIR ? (int)cluster_rank() : 0;
+  // a pair's full and tempty barriers are rank 0's
+  const uint32_t lead_full0 = PAIR ? map_to_rank(full0, 0) : full0;
+  const int first_unit = (int)blockIdx.x / kCtas, unit_step = (int)gridDim.x / kCtas;
+  const int total_units = ((p.n_tiles + kCtas - 1) / kCtas) * p.m_tiles * p.k_splits;
   JF_TL_ENTRY();
   // The next kernel may launch as soon as every CTA of this grid is resident: its CTAs take the
   // SMs this grid leaves, prefetch their own weights and park in their dependency wait, so no
@@ -408,11 +423,27 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
   // producer: initialise the barriers, then request the first weight stages right away (weights do
   // not depend on earlier kernels, so they stream in while the previous kernel finishes)
   int total_iters = 0;
-  for (int u = blockIdx.x; u < total_units; u += gridDim.x) {
+  for (int u = first_unit; u < total_units; u += unit_step) {
     const Unit w = unit_of(p, u);
     total_iters += w.kb1 - w.kb0;
   }
   const int pre = total_iters < S ? total_iters : S;
+  auto load_a = [&](const Unit& w, int kb, int s, uint64_t pol) {
+    const uint32_t dst = smem_u32(sA + s * A_STAGE_BYTES);
+    const int n0 = (w.n_tile * kCtas + rank) * kTileN;
+    if constexpr (PAIR) tma_load_2d_pair(dst, &tmA, lead_full0 + 8 * s, kb * kTileK, n0, pol);
+    else tma_load_2d(dst, &tmA, full0 + 8 * s, kb * kTileK, n0, pol);
+  };
+  auto load_b = [&](const Unit& w, int kb, int s, uint64_t pol) {
+    const uint32_t dst = smem_u32(sB + s * Cfg::B_STAGE_BYTES);
+    const int m0 = w.m_tile * BN + rank * Cfg::B_ROWS;
+    if constexpr (PAIR) tma_load_2d_pair(dst, &tmB, lead_full0 + 8 * s, kb * kTileK, m0, pol);
+    else tma_load_2d(dst, &tmB, full0 + 8 * s, kb * kTileK, m0, pol);
+  };
+  // rank 0 expects the bytes of both CTAs
+  auto expect = [&](int s) {
+    if (rank == 0) mbar_arrive_expect_tx(full0 + 8 * s, kCtas * Cfg::STAGE_BYTES);
+  };
   if (tid == 128) {
     for (int s = 0; s < S; ++s) {
       mbar_init(full0 + 8 * s, 1);
@@ -420,20 +451,24 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     }
     for (int a = 0; a < 2; ++a) {
       mbar_init(tfull0 + 8 * a, 1);
-      mbar_init(tempty0 + 8 * a, 1);
+      mbar_init(tempty0 + 8 * a, kCtas);
     }
     fence_mbar_init();
     tma_prefetch_desc(&tmA);
     tma_prefetch_desc(&tmB);
+  }
+  __syncwarp();
+  if constexpr (PAIR) cluster_sync();  // both CTAs' barriers exist
+  if (tid == 128) {
     const uint64_t polA = l2_policy_evict_first();
-    int u = blockIdx.x, kb = 0;
+    int u = first_unit, kb = 0;
     Unit w = unit_of(p, u);
     kb = w.kb0;
     for (int j = 0; j < pre; ++j) {
-      mbar_arrive_expect_tx(full0 + 8 * j, Cfg::STAGE_BYTES);
-      tma_load_2d(smem_u32(sA + j * A_STAGE_BYTES), &tmA, full0 + 8 * j, kb * kTileK, w.n_tile * kTileN, polA);
+      expect(j);
+      load_a(w, kb, j, polA);
       if (++kb == w.kb1) {
-        u += gridDim.x;
+        u += unit_step;
         if (u < total_units) {
           w = unit_of(p, u);
           kb = w.kb0;
@@ -443,11 +478,17 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
   }
   __syncwarp();
   if (warp == 4) {
-    tmem_alloc(smem_u32(tmem_slot), Cfg::TMEM_COLS);
-    tmem_relinquish();
+    if constexpr (PAIR) {
+      tmem_alloc_pair(smem_u32(tmem_slot), Cfg::TMEM_COLS);
+      tmem_relinquish_pair();
+    } else {
+      tmem_alloc(smem_u32(tmem_slot), Cfg::TMEM_COLS);
+      tmem_relinquish();
+    }
   }
   tc_fence_before();
   __syncthreads();
+  if constexpr (PAIR) cluster_sync();  // both CTAs hold their TMEM before rank 0's first MMA
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
 
@@ -457,13 +498,13 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
       pdl_wait();
       // activations of the prefetched stages
       {
-        int u = blockIdx.x;
+        int u = first_unit;
         Unit w = unit_of(p, u);
         int kb = w.kb0;
         for (int j = 0; j < pre; ++j) {
-          tma_load_2d(smem_u32(sB + j * Cfg::B_STAGE_BYTES), &tmB, full0 + 8 * j, kb * kTileK, w.m_tile * BN, polB);
+          load_b(w, kb, j, polB);
           if (++kb == w.kb1) {
-            u += gridDim.x;
+            u += unit_step;
             if (u < total_units) {
               w = unit_of(p, u);
               kb = w.kb0;
@@ -473,7 +514,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
       }
       // steady state
       int j = 0;
-      for (int u = blockIdx.x; u < total_units; u += gridDim.x) {
+      for (int u = first_unit; u < total_units; u += unit_step) {
         const Unit w = unit_of(p, u);
         bool ok = true;
         for (int kb = w.kb0; kb < w.kb1; ++kb, ++j) {
@@ -484,45 +525,74 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
             ok = false;
             break;
           }
-          mbar_arrive_expect_tx(full0 + 8 * s, Cfg::STAGE_BYTES);
-          tma_load_2d(smem_u32(sA + s * A_STAGE_BYTES), &tmA, full0 + 8 * s, kb * kTileK, w.n_tile * kTileN, polA);
-          tma_load_2d(smem_u32(sB + s * Cfg::B_STAGE_BYTES), &tmB, full0 + 8 * s, kb * kTileK, w.m_tile * BN, polB);
+          expect(s);
+          load_a(w, kb, s, polA);
+          load_b(w, kb, s, polB);
         }
         if (!ok) break;
       }
+      if constexpr (PAIR) {  // rank 0's last arrivals on this CTA's barriers, before it may leave
+        for (int q = total_iters > S ? total_iters - S : 0; q < total_iters; ++q)
+          if (!mbar_wait_bounded(empty0 + 8 * (q % S), (uint32_t)(q / S) & 1u, p.wait_ns)) break;
+      }
     }
   } else if (warp == 5) {
-    if (lane == 0) {
-      constexpr uint32_t idesc = idesc_bf16_f32(kTileN, BN);
-      int j = 0, i = 0;
+    // The whole warp walks the stages, one elected lane issues. A wait behind issued MMAs takes as long
+    // as they queue, so two stages are awaited and issued together; descriptors are a base plus constants.
+    if (rank == 0) {
+      constexpr uint32_t idesc = idesc_bf16_f32(kCtas * kTileN, BN);
+      const uint64_t da = sdesc_k_sw128(smem_u32(sA)), db = sdesc_k_sw128(smem_u32(sB));
+      int s = 0, i = 0;
+      uint32_t phase = 0;
       bool ok = true;
-      for (int u = blockIdx.x; u < total_units && ok; u += gridDim.x, ++i) {
+      for (int u = first_unit; u < total_units && ok; u += unit_step, ++i) {
         const Unit w = unit_of(p, u);
         const int acc = i & 1;
         if (i >= 2 && !mbar_wait_bounded(tempty0 + 8 * acc, (uint32_t)((i >> 1) - 1) & 1u, p.wait_ns)) {
-          jf_set_error(p.err, JF_DERR_TIMEOUT_EPI);
+          if (lane == 0) jf_set_error(p.err, JF_DERR_TIMEOUT_EPI);
           break;
         }
         tc_fence_after();
         const uint32_t dacc = tmem + (uint32_t)(acc * Cfg::ACC_COLS);
-        for (int kb = w.kb0; kb < w.kb1; ++kb, ++j) {
-          const int s = j % S;
-          if (!mbar_wait_bounded(full0 + 8 * s, (uint32_t)(j / S) & 1u, p.wait_ns)) {
-            jf_set_error(p.err, JF_DERR_TIMEOUT_TMA);
+        for (int kb = w.kb0; kb < w.kb1; kb += 2) {
+          const bool two = kb + 1 < w.kb1;
+          const int s1 = s + 1 == S ? 0 : s + 1;
+          const uint32_t phase1 = s + 1 == S ? phase ^ 1u : phase;
+          ok = mbar_wait_bounded(full0 + 8 * s, phase, p.wait_ns) &&
+               (!two || mbar_wait_bounded(full0 + 8 * s1, phase1, p.wait_ns));
+          if (!__all_sync(0xffffffffu, ok)) {
+            if (lane == 0) jf_set_error(p.err, JF_DERR_TIMEOUT_TMA);
             ok = false;
             break;
           }
           tc_fence_after();
-          const uint32_t a = smem_u32(sA + s * A_STAGE_BYTES), b = smem_u32(sB + s * Cfg::B_STAGE_BYTES);
+          if (elect_one()) {
+            auto stage_mmas = [&](int st, bool first) {
+              const uint64_t a = da + (uint64_t)(st * (A_STAGE_BYTES >> 4));
+              const uint64_t b = db + (uint64_t)(st * (Cfg::B_STAGE_BYTES >> 4));
 #pragma unroll
-          for (int kk = 0; kk < kTileK / 16; ++kk)
-            tc_mma_bf16(dacc, sdesc_k_sw128(a + kk * 32), sdesc_k_sw128(b + kk * 32), idesc,
-                        (kb > w.kb0 || kk > 0) ? 1u : 0u);
-          tc_commit(empty0 + 8 * s);
+              for (int kk = 0; kk < kTileK / 16; ++kk) {
+                const uint32_t add = (!first || kk > 0) ? 1u : 0u;
+                if constexpr (PAIR) tc_mma_bf16_pair(dacc, a + kk * 2, b + kk * 2, idesc, add);
+                else tc_mma_bf16(dacc, a + kk * 2, b + kk * 2, idesc, add);
+              }
+              if constexpr (PAIR) tc_commit_pair(empty0 + 8 * st);
+              else tc_commit(empty0 + 8 * st);
+            };
+            stage_mmas(s, kb == w.kb0);
+            if (two) stage_mmas(s1, false);
+            if (kb + 2 >= w.kb1) {
+              if constexpr (PAIR) tc_commit_pair(tfull0 + 8 * acc);
+              else tc_commit(tfull0 + 8 * acc);
+            }
+          }
+          __syncwarp();
+          s = two ? (s1 + 1 == S ? 0 : s1 + 1) : s1;
+          phase = two ? (s1 + 1 == S ? phase1 ^ 1u : phase1) : phase1;
         }
-        tc_commit(tfull0 + 8 * acc);
       }
     }
+    __syncwarp();
   } else {
     // epilogue warps 0-3
     pdl_wait();
@@ -533,7 +603,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     }
     const uint32_t lane_base = (uint32_t)(warp * 32) << 16;
     int i = 0;
-    for (int u = blockIdx.x; u < total_units; u += gridDim.x, ++i) {
+    for (int u = first_unit; u < total_units; u += unit_step, ++i) {
       const Unit w = unit_of(p, u);
       const int acc = i & 1;
       if (!mbar_wait_bounded(tfull0 + 8 * acc, (uint32_t)(i >> 1) & 1u, p.wait_ns)) {
@@ -543,15 +613,25 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
       tc_fence_after();
       const uint32_t dacc = tmem + (uint32_t)(acc * Cfg::ACC_COLS) + lane_base;
       auto get = [&](int c0, float (&v)[16]) { tmem_ld16(dacc + (uint32_t)c0, v); };
-      finish_tile<bf16, BN, EPI>(p, get, xs, sflag, w.n_tile, w.split, w.m_tile, tid, blockIdx.x, gridDim.x);
+      const int n_tile = w.n_tile * kCtas + rank;
+      if (n_tile < p.n_tiles)  // (the last pair's second tile may not exist)
+        finish_tile<bf16, BN, EPI>(p, get, xs, sflag, n_tile, w.split, w.m_tile, tid, blockIdx.x, gridDim.x);
       tc_fence_before();
       epi_sync();
-      if (tid == 0) mbar_arrive(tempty0 + 8 * acc);
+      if (tid == 0) {
+        if constexpr (PAIR) mbar_arrive_cluster(map_to_rank(tempty0 + 8 * acc, 0));
+        else mbar_arrive(tempty0 + 8 * acc);
+      }
     }
   }
   tc_fence_before();
   __syncthreads();
-  if (warp == 4) tmem_dealloc(tmem, Cfg::TMEM_COLS);
+  if constexpr (PAIR) {
+    cluster_sync();  // neither CTA leaves while the other may use its shared or tensor memory
+    if (warp == 4) tmem_dealloc_pair(tmem, Cfg::TMEM_COLS);
+  } else {
+    if (warp == 4) tmem_dealloc(tmem, Cfg::TMEM_COLS);
+  }
   JF_TL_EXIT(TL_GEMM + EPI);
 }
 
@@ -590,10 +670,8 @@ JF_DEV void f32_copy4(uint32_t dst, const float* row, int k, int K, bool ok, boo
 }
 
 JF_DEV float ld_cluster_f32(const float* p, uint32_t rank) {  // *p of the cluster's CTA `rank`
-  uint32_t addr;
   float v;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(addr) : "r"(smem_u32(p)), "r"(rank));
-  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
+  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(map_to_rank(smem_u32(p), rank)) : "memory");
   return v;
 }
 
@@ -676,46 +754,56 @@ __global__ void __launch_bounds__(F32_THREADS) k_gemm_f32(const float* __restric
   if (n_splits > 1) cluster_sync();  // the other CTAs keep their partial tiles until rank 0 has read them
 }
 
-template <int BN, int EPI>
+template <int BN, int EPI, bool PAIR>
 cudaError_t launch_tc_epi(const CUtensorMap& tmA, const CUtensorMap& tmB, const GemmParams& p, cudaStream_t st) {
-  using Cfg = TcCfg<BN>;
+  using Cfg = TcCfg<BN, PAIR>;
+  constexpr int kCtas = PAIR ? 2 : 1;
   cudaLaunchConfig_t cfg = {};
-  const int units = p.n_tiles * p.m_tiles * p.k_splits;
-  cfg.gridDim = dim3(units < p.grid ? units : p.grid);
+  const int units = ((p.n_tiles + kCtas - 1) / kCtas) * p.m_tiles * p.k_splits;
+  const int groups = p.grid / kCtas;
+  cfg.gridDim = dim3(kCtas * (units < groups ? units : groups));
   cfg.blockDim = dim3(TC_THREADS);
   cfg.dynamicSmemBytes = Cfg::SMEM;
   cfg.stream = st;
-  cudaLaunchAttribute at[1];
+  cudaLaunchAttribute at[2];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[0].val.programmaticStreamSerializationAllowed = 1;
+  at[1].id = cudaLaunchAttributeClusterDimension;
+  at[1].val.clusterDim.x = kCtas;
+  at[1].val.clusterDim.y = 1;
+  at[1].val.clusterDim.z = 1;
   cfg.attrs = at;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k_gemm_tc<BN, EPI>, tmA, tmB, p);
+  cfg.numAttrs = PAIR ? 2 : 1;
+  return cudaLaunchKernelEx(&cfg, k_gemm_tc<BN, EPI, PAIR>, tmA, tmB, p);
 }
 
-template <int BN>
+template <int BN, bool PAIR = false>
 cudaError_t launch_tc(const CUtensorMap& tmA, const CUtensorMap& tmB, const GemmParams& p, cudaStream_t st) {
   switch (p.epi.kind) {
-    case EPI_STORE: return launch_tc_epi<BN, EPI_STORE>(tmA, tmB, p, st);
-    case EPI_RESID: return launch_tc_epi<BN, EPI_RESID>(tmA, tmB, p, st);
-    case EPI_QKV: return launch_tc_epi<BN, EPI_QKV>(tmA, tmB, p, st);
-    case EPI_SWIGLU: return launch_tc_epi<BN, EPI_SWIGLU>(tmA, tmB, p, st);
-    case EPI_ARGMAX: return launch_tc_epi<BN, EPI_ARGMAX>(tmA, tmB, p, st);
-    case EPI_PARTIAL: return launch_tc_epi<BN, EPI_PARTIAL>(tmA, tmB, p, st);
+    case EPI_STORE: return launch_tc_epi<BN, EPI_STORE, PAIR>(tmA, tmB, p, st);
+    case EPI_RESID: return launch_tc_epi<BN, EPI_RESID, PAIR>(tmA, tmB, p, st);
+    case EPI_QKV: return launch_tc_epi<BN, EPI_QKV, PAIR>(tmA, tmB, p, st);
+    case EPI_SWIGLU: return launch_tc_epi<BN, EPI_SWIGLU, PAIR>(tmA, tmB, p, st);
+    case EPI_ARGMAX: return launch_tc_epi<BN, EPI_ARGMAX, PAIR>(tmA, tmB, p, st);
+    case EPI_PARTIAL: return launch_tc_epi<BN, EPI_PARTIAL, PAIR>(tmA, tmB, p, st);
     default: return cudaErrorInvalidValue;
   }
 }
 
-template <int BN>
+template <typename K>
+cudaError_t opt_in(K kernel, int smem) {
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+}
+
+template <int BN, bool PAIR = false>
 cudaError_t prep_tc() {
   cudaError_t e;
-  const int sm = TcCfg<BN>::SMEM;
-  if ((e = cudaFuncSetAttribute(k_gemm_tc<BN, EPI_STORE>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm))) return e;
-  if ((e = cudaFuncSetAttribute(k_gemm_tc<BN, EPI_RESID>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm))) return e;
-  if ((e = cudaFuncSetAttribute(k_gemm_tc<BN, EPI_QKV>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm))) return e;
-  if ((e = cudaFuncSetAttribute(k_gemm_tc<BN, EPI_SWIGLU>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm))) return e;
-  if ((e = cudaFuncSetAttribute(k_gemm_tc<BN, EPI_ARGMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm))) return e;
-  return cudaFuncSetAttribute(k_gemm_tc<BN, EPI_PARTIAL>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+  const int sm = TcCfg<BN, PAIR>::SMEM;
+  if ((e = opt_in(k_gemm_tc<BN, EPI_STORE, PAIR>, sm)) || (e = opt_in(k_gemm_tc<BN, EPI_RESID, PAIR>, sm)) ||
+      (e = opt_in(k_gemm_tc<BN, EPI_QKV, PAIR>, sm)) || (e = opt_in(k_gemm_tc<BN, EPI_SWIGLU, PAIR>, sm)) ||
+      (e = opt_in(k_gemm_tc<BN, EPI_ARGMAX, PAIR>, sm)))
+    return e;
+  return opt_in(k_gemm_tc<BN, EPI_PARTIAL, PAIR>, sm);
 }
 
 }  // namespace
@@ -744,7 +832,7 @@ static cudaError_t gemm_prepare_current() {
   if ((e = prep_tc<64>()) != cudaSuccess) return e;
   if ((e = prep_tc<128>()) != cudaSuccess) return e;
   if ((e = prep_tc<160>()) != cudaSuccess) return e;
-  return prep_tc<256>();
+  return prep_tc<256, true>();
 }
 
 // The attributes are per device: set them once for each device the process uses (outside any
@@ -775,13 +863,16 @@ int gemm_bn_for(int M) {
   return 256;
 }
 
+// Token rows of one TMA box of the activations: a pair's CTAs load half of a 256-token tile each.
+int gemm_box_rows(int bn) { return bn == 256 ? 128 : bn; }
+
 size_t gemm_smem_bytes(int bn) {
   switch (bn) {
-    case 32: return TcCfg<32>::SMEM;
-    case 64: return TcCfg<64>::SMEM;
-    case 128: return TcCfg<128>::SMEM;
-    case 160: return TcCfg<160>::SMEM;
-    default: return TcCfg<256>::SMEM;
+    case 32: return TcCfg<32, false>::SMEM;
+    case 64: return TcCfg<64, false>::SMEM;
+    case 128: return TcCfg<128, false>::SMEM;
+    case 160: return TcCfg<160, false>::SMEM;
+    default: return TcCfg<256, true>::SMEM;
   }
 }
 
@@ -792,7 +883,7 @@ cudaError_t launch_gemm_bf16(const CUtensorMap& tmA, const CUtensorMap& tmB, con
     case 64: return launch_tc<64>(tmA, tmB, p, st);
     case 128: return launch_tc<128>(tmA, tmB, p, st);
     case 160: return launch_tc<160>(tmA, tmB, p, st);
-    case 256: return launch_tc<256>(tmA, tmB, p, st);
+    case 256: return launch_tc<256, true>(tmA, tmB, p, st);
     default: return cudaErrorInvalidValue;
   }
 }

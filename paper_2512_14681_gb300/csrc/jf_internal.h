@@ -145,6 +145,7 @@ cudaError_t launch_gemm_bf16(const CUtensorMap& tmA, const CUtensorMap& tmB, con
                              cudaStream_t st);
 cudaError_t launch_gemm_f32(const float* W, const float* X, const GemmParams& p, cudaStream_t st);
 int gemm_bn_for(int M);
+int gemm_box_rows(int bn);
 #ifdef JF_TIMELINE
 // Timeline builds: point each translation unit's record buffer / counter at caller memory.
 cudaError_t tl_set_gemm(void* records, void* counter);
