@@ -93,22 +93,30 @@ JF_DEV void fence_mbar_init() { asm volatile("fence.mbarrier_init.release.cluste
 
 JF_DEV void fence_proxy_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
-JF_DEV void mbar_arrive_expect_tx(uint32_t bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+// (predicated off when `on` is false, like the copies below)
+JF_DEV void mbar_arrive_expect_tx(uint32_t bar, uint32_t bytes, bool on = true) {
+  asm volatile(
+      "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %2, 0;\n\t"
+      "@q mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n\t}" ::"r"(bar),
+      "r"(bytes), "r"((int)on)
+      : "memory");
 }
 
 JF_DEV void mbar_arrive(uint32_t bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 
+// True once phase `parity` is complete. The thread may be suspended for up to kWaitHintNs meanwhile: a
+// wait that polls takes issue slots from the warps that feed it.
+constexpr uint32_t kWaitHintNs = 20000u;
 JF_DEV bool mbar_try_wait(uint32_t bar, uint32_t parity) {
   uint32_t ok;
   asm volatile(
       "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
       "selp.u32 %0, 1, 0, p;\n\t}"
       : "=r"(ok)
-      : "r"(bar), "r"(parity)
+      : "r"(bar), "r"(parity), "r"(kWaitHintNs)
       : "memory");
   return ok != 0;
 }
@@ -162,11 +170,12 @@ JF_DEV uint64_t l2_policy_evict_last() {
 // 2-D tiled load: box at coordinates (c0 = innermost, c1) into shared memory, completing
 // `bytes` on mbarrier `bar`. The innermost coordinate is always a multiple of 64 elements
 // (128 bytes) here, which keeps every copy on a 16-byte boundary.
-JF_DEV void tma_load_2d(uint32_t smem_dst, const void* tmap, uint32_t bar, int c0, int c1, uint64_t policy) {
+JF_DEV void tma_load_2d(uint32_t smem_dst, const void* tmap, uint32_t bar, int c0, int c1, uint64_t policy, bool on) {
   asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint"
-      " [%0], [%1, {%2, %3}], [%4], %5;" ::"r"(smem_dst),
-      "l"(tmap), "r"(c0), "r"(c1), "r"(bar), "l"(policy)
+      "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %6, 0;\n\t"
+      "@q cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint"
+      " [%0], [%1, {%2, %3}], [%4], %5;\n\t}" ::"r"(smem_dst),
+      "l"(tmap), "r"(c0), "r"(c1), "r"(bar), "l"(policy), "r"((int)on)
       : "memory");
 }
 
@@ -187,11 +196,13 @@ JF_DEV void tma_load_3d_plain(uint32_t smem_dst, const void* tmap, uint32_t bar,
 
 // 2-D tiled load by a CTA of a pair (cta_group::2): into its own shared memory, completing on an
 // mbarrier of either CTA (a shared::cluster address).
-JF_DEV void tma_load_2d_pair(uint32_t smem_dst, const void* tmap, uint32_t bar, int c0, int c1, uint64_t policy) {
+JF_DEV void tma_load_2d_pair(uint32_t smem_dst, const void* tmap, uint32_t bar, int c0, int c1, uint64_t policy,
+                             bool on) {
   asm volatile(
-      "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint"
-      " [%0], [%1, {%2, %3}], [%4], %5;" ::"r"(smem_dst),
-      "l"(tmap), "r"(c0), "r"(c1), "r"(bar), "l"(policy)
+      "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %6, 0;\n\t"
+      "@q cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint"
+      " [%0], [%1, {%2, %3}], [%4], %5;\n\t}" ::"r"(smem_dst),
+      "l"(tmap), "r"(c0), "r"(c1), "r"(bar), "l"(policy), "r"((int)on)
       : "memory");
 }
 

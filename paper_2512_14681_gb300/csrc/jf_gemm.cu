@@ -32,7 +32,8 @@ struct TcCfg {
   static constexpr int B_STAGE_BYTES = B_ROWS * kTileK * 2;
   static constexpr int STAGE_BYTES = A_STAGE_BYTES + B_STAGE_BYTES;
   static constexpr int S0 = (SMEM_LIMIT - 1024 - EPI_STAGE_BYTES - 512) / STAGE_BYTES;
-  static constexpr int STAGES = S0 < 2 ? 2 : (S0 > 12 ? 12 : S0);
+  static constexpr int STAGES = S0 > 12 ? 12 : S0 / 2 * 2;  // two 64-k blocks a stage pair
+  static_assert(STAGES >= 4, "at least two stage pairs");
   static constexpr int ACC_COLS = BN;   // one accumulator; two are allocated (double buffer)
   static constexpr int TMEM_COLS = 2 * BN <= 32 ? 32 : (2 * BN <= 64 ? 64 : (2 * BN <= 128 ? 128 : (2 * BN <= 256 ? 256 : 512)));
   static constexpr int SMEM = 1024 + STAGES * STAGE_BYTES + EPI_STAGE_BYTES + 512;
@@ -372,15 +373,14 @@ JF_DEV Unit unit_of(const GemmParams& p, int u) {
   const int t = u / p.k_splits;
   w.m_tile = t % p.m_tiles;
   w.n_tile = t / p.m_tiles;
-  w.kb0 = (int)(((long long)p.kb_total * w.split) / p.k_splits);
-  w.kb1 = (int)(((long long)p.kb_total * (w.split + 1)) / p.k_splits);
+  w.kb0 = (int)((unsigned)(p.kb_total * w.split) / (unsigned)p.k_splits);  // (at most 8 splits)
+  w.kb1 = (int)((unsigned)(p.kb_total * (w.split + 1)) / (unsigned)p.k_splits);
   return w;
 }
 
 // ---------------------------------------------------------------------------------------------
 // bf16 tcgen05 persistent kernel, 192 threads: warps 0-3 epilogue (warp w reads TMEM lanes
-// 32w .. 32w+31), warp 4 lane 0 = TMA producer (warp 4 also owns the TMEM allocation),
-// warp 5 = MMA issuer.
+// 32w .. 32w+31), warp 4 = TMA producer, warp 5 = MMA issuer (and the TMEM allocation).
 //
 // PAIR (256-token tiles, i.e. more than 160 rows): two CTAs on neighbouring SMs take a tile of 256
 // weight rows together (cta_group::2). Each loads its own 128 weight rows and half of the tokens (32 KB
@@ -395,7 +395,9 @@ template <int BN, int EPI, bool PAIR>
 __global__ void __launch_bounds__(TC_THREADS, 1)
     k_gemm_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const GemmParams p) {
   using Cfg = TcCfg<BN, PAIR>;
-  constexpr int S = Cfg::STAGES;
+  // The ring's unit is a stage pair: two 64-k blocks (one at an odd unit's end) with one full and one
+  // empty barrier, so that a wait, an arrival and a commit (about 100-200 cycles each) serve 128 k.
+  constexpr int S = Cfg::STAGES, D = S / 2;
   constexpr int kCtas = PAIR ? 2 : 1;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = align1024(smem_raw);
@@ -403,12 +405,14 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
   uint8_t* sB = smem + S * A_STAGE_BYTES;
   float* xs = reinterpret_cast<float*>(sB + S * Cfg::B_STAGE_BYTES);
   uint64_t* bars = reinterpret_cast<uint64_t*>(reinterpret_cast<uint8_t*>(xs) + EPI_STAGE_BYTES);
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * S + 4);
+  const uint32_t idle = smem_u32(bars + 2 * D + 4);  // never completes: a wait for its odd phase passes
+  const uint32_t sink = smem_u32(bars + 2 * D + 5);  // nobody waits for it
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * D + 6);
   int* sflag = reinterpret_cast<int*>(tmem_slot + 1);
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const uint32_t full0 = smem_u32(bars), empty0 = smem_u32(bars + S);
-  const uint32_t tfull0 = smem_u32(bars + 2 * S), tempty0 = smem_u32(bars + 2 * S + 2);
+  const uint32_t full0 = smem_u32(bars), empty0 = smem_u32(bars + D);
+  const uint32_t tfull0 = smem_u32(bars + 2 * D), tempty0 = smem_u32(bars + 2 * D + 2);
   const int rank = PAIR ? (int)cluster_rank() : 0;
   // a pair's full and tempty barriers are rank 0's
   const uint32_t lead_full0 = PAIR ? map_to_rank(full0, 0) : full0;
@@ -420,64 +424,53 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
   // launch latency is paid after the last tile (it writes nothing before that wait).
   pdl_launch_dependents();
 
-  // producer: initialise the barriers, then request the first weight stages right away (weights do
-  // not depend on earlier kernels, so they stream in while the previous kernel finishes)
-  int total_iters = 0;
+  int total_iters = 0;  // stage pairs of this CTA
   for (int u = first_unit; u < total_units; u += unit_step) {
     const Unit w = unit_of(p, u);
-    total_iters += w.kb1 - w.kb0;
+    total_iters += (w.kb1 - w.kb0 + 1) / 2;
   }
-  const int pre = total_iters < S ? total_iters : S;
-  auto load_a = [&](const Unit& w, int kb, int s, uint64_t pol) {
-    const uint32_t dst = smem_u32(sA + s * A_STAGE_BYTES);
+  const int pre = total_iters < D ? total_iters : D;
+  // k blocks kb and kb + 1 (if it belongs to the unit) into stage pair d (predicated off when `on` is false)
+  auto load_a = [&](const Unit& w, int kb, int d, uint64_t pol, bool on) {
     const int n0 = (w.n_tile * kCtas + rank) * kTileN;
-    if constexpr (PAIR) tma_load_2d_pair(dst, &tmA, lead_full0 + 8 * s, kb * kTileK, n0, pol);
-    else tma_load_2d(dst, &tmA, full0 + 8 * s, kb * kTileK, n0, pol);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const uint32_t dst = smem_u32(sA + (2 * d + h) * A_STAGE_BYTES);
+      const bool live = on && kb + h < w.kb1;
+      if constexpr (PAIR) tma_load_2d_pair(dst, &tmA, lead_full0 + 8 * d, (kb + h) * kTileK, n0, pol, live);
+      else tma_load_2d(dst, &tmA, full0 + 8 * d, (kb + h) * kTileK, n0, pol, live);
+    }
   };
-  auto load_b = [&](const Unit& w, int kb, int s, uint64_t pol) {
-    const uint32_t dst = smem_u32(sB + s * Cfg::B_STAGE_BYTES);
+  auto load_b = [&](const Unit& w, int kb, int d, uint64_t pol, bool on) {
     const int m0 = w.m_tile * BN + rank * Cfg::B_ROWS;
-    if constexpr (PAIR) tma_load_2d_pair(dst, &tmB, lead_full0 + 8 * s, kb * kTileK, m0, pol);
-    else tma_load_2d(dst, &tmB, full0 + 8 * s, kb * kTileK, m0, pol);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const uint32_t dst = smem_u32(sB + (2 * d + h) * Cfg::B_STAGE_BYTES);
+      const bool live = on && kb + h < w.kb1;
+      if constexpr (PAIR) tma_load_2d_pair(dst, &tmB, lead_full0 + 8 * d, (kb + h) * kTileK, m0, pol, live);
+      else tma_load_2d(dst, &tmB, full0 + 8 * d, (kb + h) * kTileK, m0, pol, live);
+    }
   };
   // rank 0 expects the bytes of both CTAs
-  auto expect = [&](int s) {
-    if (rank == 0) mbar_arrive_expect_tx(full0 + 8 * s, kCtas * Cfg::STAGE_BYTES);
+  auto expect = [&](const Unit& w, int kb, int d, bool on) {
+    mbar_arrive_expect_tx(full0 + 8 * d, (kb + 1 < w.kb1 ? 2 : 1) * kCtas * Cfg::STAGE_BYTES, on && rank == 0);
   };
   if (tid == 128) {
-    for (int s = 0; s < S; ++s) {
-      mbar_init(full0 + 8 * s, 1);
-      mbar_init(empty0 + 8 * s, 1);
+    for (int d = 0; d < D; ++d) {
+      mbar_init(full0 + 8 * d, 1);
+      mbar_init(empty0 + 8 * d, 1);
     }
     for (int a = 0; a < 2; ++a) {
       mbar_init(tfull0 + 8 * a, 1);
       mbar_init(tempty0 + 8 * a, kCtas);
     }
+    mbar_init(idle, 1);
+    mbar_init(sink, 1);
     fence_mbar_init();
     tma_prefetch_desc(&tmA);
     tma_prefetch_desc(&tmB);
   }
-  __syncwarp();
-  if constexpr (PAIR) cluster_sync();  // both CTAs' barriers exist
-  if (tid == 128) {
-    const uint64_t polA = l2_policy_evict_first();
-    int u = first_unit, kb = 0;
-    Unit w = unit_of(p, u);
-    kb = w.kb0;
-    for (int j = 0; j < pre; ++j) {
-      expect(j);
-      load_a(w, kb, j, polA);
-      if (++kb == w.kb1) {
-        u += unit_step;
-        if (u < total_units) {
-          w = unit_of(p, u);
-          kb = w.kb0;
-        }
-      }
-    }
-  }
-  __syncwarp();
-  if (warp == 4) {
+  if (warp == 5) {
     if constexpr (PAIR) {
       tmem_alloc_pair(smem_u32(tmem_slot), Cfg::TMEM_COLS);
       tmem_relinquish_pair();
@@ -486,63 +479,92 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
       tmem_relinquish();
     }
   }
+  __syncwarp();
   tc_fence_before();
-  __syncthreads();
-  if constexpr (PAIR) cluster_sync();  // both CTAs hold their TMEM before rank 0's first MMA
+  if constexpr (PAIR) {
+    __syncthreads();
+    cluster_sync();  // both CTAs' barriers exist, and both hold their TMEM
+  } else if (warp == 4) {
+    asm volatile("bar.arrive 2, 192;" ::: "memory");  // the producer starts without waiting for the others
+  } else {
+    asm volatile("bar.sync 2, 192;" ::: "memory");
+  }
   tc_fence_after();
-  const uint32_t tmem = *tmem_slot;
 
   if (warp == 4) {
-    if (lane == 0) {
-      const uint64_t polA = l2_policy_evict_first(), polB = l2_policy_evict_last();
-      pdl_wait();
-      // activations of the prefetched stages
-      {
-        int u = first_unit;
-        Unit w = unit_of(p, u);
-        int kb = w.kb0;
-        for (int j = 0; j < pre; ++j) {
-          load_b(w, kb, j, polB);
-          if (++kb == w.kb1) {
-            u += unit_step;
-            if (u < total_units) {
-              w = unit_of(p, u);
-              kb = w.kb0;
-            }
-          }
-        }
+    // Stage pairs 0 .. pre-1: lane j requests the weights of pair j before the dependency wait (they do
+    // not depend on earlier kernels, so they stream in while the previous kernel finishes) and its
+    // activations right after it; from then on one lane requests both of a pair as it comes free. Round
+    // -1 of the loop goes through all of it with the requests predicated off, so that the code is in the
+    // instruction cache when the wait ends: the weights that stream through L2 push code out of it, and
+    // fetching it there put the first refill 2.5 us after the wait (now 0.8).
+    const uint64_t polA = l2_policy_evict_first(), polB = l2_policy_evict_last();
+    Unit w0 = unit_of(p, first_unit);
+    int u = first_unit, kb0 = w0.kb0 + 2 * lane;  // stage pair `lane`
+    while (lane < pre && kb0 >= w0.kb1) {
+      u += unit_step;
+      const int over = kb0 - (w0.kb1 + ((w0.kb1 - w0.kb0) & 1));  // (a unit takes whole pairs)
+      w0 = unit_of(p, u);
+      kb0 = w0.kb0 + over;
+    }
+    if (lane < pre) {
+      expect(w0, kb0, lane, true);
+      load_a(w0, kb0, lane, polA, true);
+    }
+    __syncwarp();
+    u = __shfl_sync(0xffffffffu, u, pre - 1);
+    int kb = __shfl_sync(0xffffffffu, kb0, pre - 1) + 2;
+    Unit w = unit_of(p, u);
+    int d = pre == D ? 0 : pre;
+    uint32_t parity = 0u;
+#pragma unroll 1
+    for (int q = -1; q <= 0 || pre + q < total_iters; ++q) {
+      const bool on = q >= 0;
+      if (q <= 0) {
+        if (on) pdl_wait();
+        if (lane < pre) load_b(w0, kb0, lane, polB, on);
+        __syncwarp();
+        if (on && pre >= total_iters) break;
       }
-      // steady state
-      int j = 0;
-      for (int u = first_unit; u < total_units; u += unit_step) {
-        const Unit w = unit_of(p, u);
-        bool ok = true;
-        for (int kb = w.kb0; kb < w.kb1; ++kb, ++j) {
-          if (j < pre) continue;
-          const int s = j % S;
-          if (!mbar_wait_bounded(empty0 + 8 * s, (uint32_t)((j / S) - 1) & 1u, p.wait_ns)) {
-            jf_set_error(p.err, JF_DERR_TIMEOUT_MMA);
-            ok = false;
-            break;
-          }
-          expect(s);
-          load_a(w, kb, s, polA);
-          load_b(w, kb, s, polB);
-        }
-        if (!ok) break;
+      if (on && kb >= w.kb1) {
+        u += unit_step;
+        w = unit_of(p, u);
+        kb = w.kb0;
       }
-      if constexpr (PAIR) {  // rank 0's last arrivals on this CTA's barriers, before it may leave
-        for (int q = total_iters > S ? total_iters - S : 0; q < total_iters; ++q)
-          if (!mbar_wait_bounded(empty0 + 8 * (q % S), (uint32_t)(q / S) & 1u, p.wait_ns)) break;
+      const bool ok = mbar_wait_bounded(on ? empty0 + 8 * d : idle, on ? parity : 1u, p.wait_ns);
+      if (!__all_sync(0xffffffffu, ok)) {
+        if (lane == 0) jf_set_error(p.err, JF_DERR_TIMEOUT_MMA);
+        break;
+      }
+      if (elect_one()) {
+        expect(w, kb, d, on);
+        load_a(w, kb, d, polA, on);
+        load_b(w, kb, d, polB, on);
+      }
+      __syncwarp();
+      if (on) {
+        kb += 2;
+        if (++d == D) {
+          d = 0;
+          parity ^= 1u;
+        }
       }
     }
+    if constexpr (PAIR) {  // rank 0's last arrivals on this CTA's barriers, before it may leave
+      for (int q = total_iters > D ? total_iters - D : 0; q < total_iters; ++q)
+        if (!mbar_wait_bounded(empty0 + 8 * (q % D), (uint32_t)(q / D) & 1u, p.wait_ns)) break;
+    }
+    __syncwarp();
   } else if (warp == 5) {
-    // The whole warp walks the stages, one elected lane issues. A wait behind issued MMAs takes as long
-    // as they queue, so two stages are awaited and issued together; descriptors are a base plus constants.
+    // The whole warp walks the stage pairs, one elected lane issues (a wait behind issued MMAs takes as
+    // long as they queue); descriptors are a base plus constants. The first pass over the loop computes
+    // on whatever the stages hold, into an accumulator that the first real MMA overwrites, and its waits
+    // pass: it fetches the code while the stages are on their way.
+    const uint32_t tmem = *tmem_slot;
     if (rank == 0) {
       constexpr uint32_t idesc = idesc_bf16_f32(kCtas * kTileN, BN);
       const uint64_t da = sdesc_k_sw128(smem_u32(sA)), db = sdesc_k_sw128(smem_u32(sB));
-      int s = 0, i = 0;
+      int d = 0, i = 0;
       uint32_t phase = 0;
       bool ok = true;
       for (int u = first_unit; u < total_units && ok; u += unit_step, ++i) {
@@ -554,12 +576,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         }
         tc_fence_after();
         const uint32_t dacc = tmem + (uint32_t)(acc * Cfg::ACC_COLS);
-        for (int kb = w.kb0; kb < w.kb1; kb += 2) {
-          const bool two = kb + 1 < w.kb1;
-          const int s1 = s + 1 == S ? 0 : s + 1;
-          const uint32_t phase1 = s + 1 == S ? phase ^ 1u : phase;
-          ok = mbar_wait_bounded(full0 + 8 * s, phase, p.wait_ns) &&
-               (!two || mbar_wait_bounded(full0 + 8 * s1, phase1, p.wait_ns));
+#pragma unroll 1
+        for (int kb = w.kb0 - (i == 0 ? 2 : 0); kb < w.kb1; kb += 2) {
+          const bool on = kb >= w.kb0;  // (a unit has at least one k block: the last round is on)
+          ok = mbar_wait_bounded(on ? full0 + 8 * d : idle, on ? phase : 1u, p.wait_ns);
           if (!__all_sync(0xffffffffu, ok)) {
             if (lane == 0) jf_set_error(p.err, JF_DERR_TIMEOUT_TMA);
             ok = false;
@@ -567,28 +587,32 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
           }
           tc_fence_after();
           if (elect_one()) {
-            auto stage_mmas = [&](int st, bool first) {
-              const uint64_t a = da + (uint64_t)(st * (A_STAGE_BYTES >> 4));
-              const uint64_t b = db + (uint64_t)(st * (Cfg::B_STAGE_BYTES >> 4));
+            const uint64_t a0 = da + (uint64_t)(d * (2 * A_STAGE_BYTES >> 4));
+            const uint64_t b0 = db + (uint64_t)(d * (2 * Cfg::B_STAGE_BYTES >> 4));
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+              if (h == 1 && kb + 1 >= w.kb1) break;
 #pragma unroll
               for (int kk = 0; kk < kTileK / 16; ++kk) {
-                const uint32_t add = (!first || kk > 0) ? 1u : 0u;
-                if constexpr (PAIR) tc_mma_bf16_pair(dacc, a + kk * 2, b + kk * 2, idesc, add);
-                else tc_mma_bf16(dacc, a + kk * 2, b + kk * 2, idesc, add);
+                const uint64_t a = a0 + h * (A_STAGE_BYTES >> 4) + kk * 2, b = b0 + h * (Cfg::B_STAGE_BYTES >> 4) + kk * 2;
+                const uint32_t add = (h > 0 || kk > 0 || kb != w.kb0) ? 1u : 0u;
+                if constexpr (PAIR) tc_mma_bf16_pair(dacc, a, b, idesc, add);
+                else tc_mma_bf16(dacc, a, b, idesc, add);
               }
-              if constexpr (PAIR) tc_commit_pair(empty0 + 8 * st);
-              else tc_commit(empty0 + 8 * st);
-            };
-            stage_mmas(s, kb == w.kb0);
-            if (two) stage_mmas(s1, false);
+            }
+            const uint32_t bar = on ? empty0 + 8 * d : sink;
+            if constexpr (PAIR) tc_commit_pair(bar);
+            else tc_commit(bar);
             if (kb + 2 >= w.kb1) {
               if constexpr (PAIR) tc_commit_pair(tfull0 + 8 * acc);
               else tc_commit(tfull0 + 8 * acc);
             }
           }
           __syncwarp();
-          s = two ? (s1 + 1 == S ? 0 : s1 + 1) : s1;
-          phase = two ? (s1 + 1 == S ? phase1 ^ 1u : phase1) : phase1;
+          if (on && ++d == D) {
+            d = 0;
+            phase ^= 1u;
+          }
         }
       }
     }
@@ -601,6 +625,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
       argmax_init_slots(p.epi, 0, p.M, blockIdx.x, gridDim.x, tid, 128);
       epi_sync();
     }
+    const uint32_t tmem = *tmem_slot;
     const uint32_t lane_base = (uint32_t)(warp * 32) << 16;
     int i = 0;
     for (int u = first_unit; u < total_units; u += unit_step, ++i) {
@@ -628,9 +653,9 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
   __syncthreads();
   if constexpr (PAIR) {
     cluster_sync();  // neither CTA leaves while the other may use its shared or tensor memory
-    if (warp == 4) tmem_dealloc_pair(tmem, Cfg::TMEM_COLS);
+    if (warp == 5) tmem_dealloc_pair(*tmem_slot, Cfg::TMEM_COLS);
   } else {
-    if (warp == 4) tmem_dealloc(tmem, Cfg::TMEM_COLS);
+    if (warp == 5) tmem_dealloc(*tmem_slot, Cfg::TMEM_COLS);
   }
   JF_TL_EXIT(TL_GEMM + EPI);
 }
