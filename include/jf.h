@@ -276,7 +276,7 @@ jf_status jf_wait_limit_probe(jf_ctx* ctx, uint64_t* waited_ns);
  * counter: a device int32 the caller zeroes, incremented once per record (records past the
  * maximum are dropped). Kernel ids: 1 RMSNorm, 2 RMSNorm adding split-K partials, 3 QKV finish,
  * 5 attention, 10 + e projection GEMM with epilogue e (13 SwiGLU, 14 argmax, 15 split-K partials),
- * 20 embedding, 21 acceptance, 22 KV commit. (NULL, NULL) stops recording. Not tied to a context:
+ * 20 embedding, 21 acceptance, 22 KV commit, 23 argmax over the LM head's slots. (NULL, NULL) stops recording. Not tied to a context:
  * the setting is process-wide and reaches CUDA graphs captured before it. */
 #define JF_TL_MAX_RECORDS 2000000
 jf_status jf_tl_enable(void* records, void* counter);

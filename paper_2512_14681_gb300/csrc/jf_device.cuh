@@ -26,7 +26,7 @@ JF_DEV uint64_t jf_globaltimer() {
 // Kernel ids of the timeline records.
 enum TlKernel : unsigned {
   TL_NORM = 1, TL_NORM_ACC = 2, TL_QKV_FINISH = 3, TL_ATTN = 5, TL_GEMM = 10 /* + epilogue kind */,
-  TL_EMBED = 20, TL_ACCEPT = 21, TL_COMMIT = 22
+  TL_EMBED = 20, TL_ACCEPT = 21, TL_COMMIT = 22, TL_ARGMAX = 23
 };
 
 // Timeline of the forward's kernels, compiled in only with -DJF_TIMELINE (the default build has
@@ -381,6 +381,3 @@ JF_DEV float warp_sum(float v) {
 }
 
 JF_DEV float silu_f(float x) { return x / (1.0f + __expf(-x)); }
-
-// (value, index) ordering of the greedy decision: larger value wins, lower index on ties.
-JF_DEV bool better(float v, int i, float bv, int bi) { return v > bv || (v == bv && i < bi); }

@@ -50,12 +50,115 @@ JF_DEV uint8_t* align1024(uint8_t* p) {
 }
 
 // ---------------------------------------------------------------------------------------------
+// Greedy argmax. Logits are compared through keys that preserve their order as unsigned integers (-0
+// counts as +0, NaN as the lowest, key 0). Every CTA keeps a running entry (best key, its lowest index,
+// runner-up key) of every row over the vocabulary tiles it takes: in shared memory for up to
+// kAmTableRows rows, otherwise in its global slot; k_argmax_finish merges the CTAs' slots. The merge is
+// associative and commutative, so the result does not depend on which CTA took which tile. With
+// 15 shuffles a column and the entries in global memory the epilogue, not the weights, set the pace of
+// the LM head above 32 rows, and one CTA merged all slots at the end (8 layers and head of the 7B shape,
+// 32 rows 941 -> 929 us, 160 rows 1286 -> 1189, 512 rows 2427 -> 2072; 1.5B, 64 rows 499 -> 449).
+// ---------------------------------------------------------------------------------------------
+JF_DEV uint32_t am_key(float v) {
+  const uint32_t u = __float_as_uint(v + 0.0f);
+  return v != v ? 0u : ((u & 0x80000000u) ? ~u : (u | 0x80000000u));
+}
+JF_DEV float am_value(uint32_t key) { return __uint_as_float((key & 0x80000000u) ? key ^ 0x80000000u : ~key); }
+JF_DEV void am_merge(uint32_t& b1, uint32_t& bi, uint32_t& b2, uint32_t o1, uint32_t oi, uint32_t o2) {
+  if (o1 > b1 || (o1 == b1 && oi < bi)) {
+    b2 = b1 > o2 ? b1 : o2;
+    b1 = o1;
+    bi = oi;
+  } else {
+    b2 = b2 > o1 ? b2 : o1;
+  }
+}
+
+constexpr int kAmRedWords = 2 * 4 * 16 * 3;  // [chunk parity][warp][column][3]
+constexpr int kAmTableRows = 512;
+static_assert((kAmRedWords + 3 * kAmTableRows) * 4 <= EPI_STAGE_BYTES, "argmax tables fit the epilogue's staging");
+constexpr uint32_t kAmNoIndex = 0x7fffffffu;
+
+// Running entries of a CTA: entry of row m at [m * stride].
+struct AmEntries {
+  uint32_t *red, *k1, *idx, *k2;
+  size_t stride;
+};
+JF_DEV AmEntries am_global(const GemmEpi& e, uint32_t* red, int slot, int n_slots) {
+  return AmEntries{red, reinterpret_cast<uint32_t*>(e.am_v1) + slot, reinterpret_cast<uint32_t*>(e.am_i1) + slot,
+                   reinterpret_cast<uint32_t*>(e.am_v2) + slot, (size_t)n_slots};
+}
+JF_DEV AmEntries am_shared(uint32_t* words) {
+  uint32_t* t = words + kAmRedWords;
+  return AmEntries{words, t, t + kAmTableRows, t + 2 * kAmTableRows, 1};
+}
+JF_DEV void am_clear(const AmEntries& am, int m_begin, int m_end, int tid, int nthreads) {
+  for (int m = m_begin + tid; m < m_end; m += nthreads) {
+    am.k1[m * am.stride] = 0u;
+    am.idx[m * am.stride] = kAmNoIndex;
+    am.k2[m * am.stride] = 0u;
+  }
+}
+
+// One warp per row: the slots of all CTAs, eight a lane in flight.
+__global__ void __launch_bounds__(128) k_argmax_finish(const uint32_t* k1, const uint32_t* idx, const uint32_t* k2,
+                                                       int n_slots, int M, int* out, float* top2) {
+  JF_TL_ENTRY();
+  pdl_launch_dependents();
+  const int m = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  pdl_wait();
+  JF_TL_WAITED();
+  if (m < M) {
+    uint32_t b1 = 0, bi = kAmNoIndex, b2 = 0;
+    for (int s0 = 0; s0 < n_slots; s0 += 8 * 32) {
+      uint32_t a[8], i[8], c[8];
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        const int s = s0 + 32 * k + lane;
+        const size_t at = (size_t)m * n_slots + s;
+        a[k] = s < n_slots ? __ldcg(k1 + at) : 0u;
+        i[k] = s < n_slots ? __ldcg(idx + at) : kAmNoIndex;
+        c[k] = s < n_slots ? __ldcg(k2 + at) : 0u;
+      }
+#pragma unroll
+      for (int k = 0; k < 8; ++k) am_merge(b1, bi, b2, a[k], i[k], c[k]);
+    }
+    const uint32_t top = __reduce_max_sync(0xffffffffu, b1);
+    const uint32_t best = __reduce_min_sync(0xffffffffu, b1 == top ? bi : 0xffffffffu);
+    const uint32_t second = __reduce_max_sync(0xffffffffu, (b1 == top && bi == best) ? b2 : b1);
+    if (lane == 0) {
+      out[m] = (int)best;
+      if (top2) {
+        top2[2 * m] = am_value(top);
+        top2[2 * m + 1] = am_value(second);
+      }
+    }
+  }
+  JF_TL_EXIT(TL_ARGMAX);
+}
+
+cudaError_t launch_argmax_finish(const GemmEpi& e, int M, int n_slots, cudaStream_t st) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((M + 3) / 4);
+  cfg.blockDim = dim3(128);
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, k_argmax_finish, reinterpret_cast<const uint32_t*>(e.am_v1),
+                            reinterpret_cast<const uint32_t*>(e.am_i1), reinterpret_cast<const uint32_t*>(e.am_v2), n_slots,
+                            M, e.am_out, e.top2_out);
+}
+
+// ---------------------------------------------------------------------------------------------
 // Epilogue on one 16-column chunk: thread `row` (0..127) holds v[j] = Y[m0 + c0 + j, n0 + row].
 // xs: shared staging [16][128] fp32 (exchange between the two halves of a tile).
 // ---------------------------------------------------------------------------------------------
 template <typename T, int EPI>
 JF_DEV void epilogue_chunk(const GemmEpi& e, const float (&v)[16], int row, int n0, int m0, int c0, float* xs,
-                           int n_tile, int slot, int n_slots) {
+                           int n_tile, const AmEntries& am) {
   const int n = n0 + row;
   constexpr int kind = EPI;
   if constexpr (kind == EPI_STORE || kind == EPI_RESID) {
@@ -142,136 +245,58 @@ JF_DEV void epilogue_chunk(const GemmEpi& e, const float (&v)[16], int row, int 
     epi_sync();
     return;
   } else {
-    // EPI_ARGMAX: best (value, index) and runner-up value over this tile's 128 vocabulary rows
-    float* red = xs;  // [4 warps][16 cols][3]
+    // EPI_ARGMAX: best (value, lowest index) and runner-up over this tile's 128 vocabulary rows. A warp
+    // reduces a column with two redux instructions on order-preserving keys; lane j keeps column j.
     const int warp = row >> 5, lane = row & 31;
+    uint32_t b1 = 0, b2 = 0, bi = 0;
 #pragma unroll
     for (int j = 0; j < 16; ++j) {
-      float b1 = (n < e.N) ? v[j] : -INFINITY;
-      int bi = (n < e.N) ? n : 0x7fffffff;
-      float b2 = -INFINITY;
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        const float o1 = __shfl_xor_sync(0xffffffffu, b1, o);
-        const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-        const float o2 = __shfl_xor_sync(0xffffffffu, b2, o);
-        if (better(o1, oi, b1, bi)) { b2 = fmaxf(b1, o2); b1 = o1; bi = oi; }
-        else { b2 = fmaxf(b2, o1); }
-      }
-      if (lane == 0) {
-        red[(warp * 16 + j) * 3 + 0] = b1;
-        red[(warp * 16 + j) * 3 + 1] = __int_as_float(bi);
-        red[(warp * 16 + j) * 3 + 2] = b2;
+      const uint32_t key = n < e.N ? am_key(v[j]) : 0u;
+      const uint32_t top = __reduce_max_sync(0xffffffffu, key);
+      const int win = __ffs((int)__ballot_sync(0xffffffffu, key == top)) - 1;
+      const uint32_t second = __reduce_max_sync(0xffffffffu, lane == win ? 0u : key);
+      if (lane == j) {
+        b1 = top;
+        bi = (uint32_t)(n - lane + win);
+        b2 = second;
       }
     }
+    uint32_t* red = am.red + ((c0 >> 4) & 1) * (4 * 16 * 3);  // alternates: one barrier a chunk is enough
+    if (lane < 16) {
+      uint32_t* mine = red + (warp * 16 + lane) * 3;
+      mine[0] = b1;
+      mine[1] = bi;
+      mine[2] = b2;
+    }
     epi_sync();
-    if (row < 16) {
-      const int j = row, m = m0 + c0 + j;
-      float b1 = red[j * 3 + 0], b2 = red[j * 3 + 2];
-      int bi = __float_as_int(red[j * 3 + 1]);
+    const int m = m0 + c0 + row;
+    if (row < 16 && m < e.M) {
+#pragma unroll
       for (int w = 1; w < 4; ++w) {
-        const float o1 = red[(w * 16 + j) * 3 + 0], o2 = red[(w * 16 + j) * 3 + 2];
-        const int oi = __float_as_int(red[(w * 16 + j) * 3 + 1]);
-        if (better(o1, oi, b1, bi)) { b2 = fmaxf(b1, o2); b1 = o1; bi = oi; }
-        else { b2 = fmaxf(b2, o1); }
+        const uint32_t* o = red + (w * 16 + row) * 3;
+        am_merge(b1, bi, b2, o[0], o[1], o[2]);
       }
-      if (m < e.M) {
-        // fold this tile into the CTA's running (best, index, runner-up) of row m; the same
-        // thread owns the slot for every tile of the CTA, so program order orders the updates
-        const size_t at = (size_t)m * n_slots + slot;
-        const float o1 = e.am_v1[at], o2 = e.am_v2[at];
-        const int oi = e.am_i1[at];
-        if (better(b1, bi, o1, oi)) {
-          e.am_v1[at] = b1;
-          e.am_i1[at] = bi;
-          e.am_v2[at] = fmaxf(o1, b2);
-        } else {
-          e.am_v2[at] = fmaxf(o2, b1);
-        }
-      }
-    }
-    epi_sync();
-  }
-}
-
-// Argmax partials: slot (m, s) holds CTA s's running (best value, its index, runner-up value) of
-// row m over the vocabulary tiles that CTA has folded in. Every CTA starts its slots empty.
-JF_DEV void argmax_init_slots(const GemmEpi& e, int m_begin, int m_end, int slot, int n_slots, int tid, int nthreads) {
-  if (m_end > e.M) m_end = e.M;
-  for (int m = m_begin + tid; m < m_end; m += nthreads) {
-    const size_t at = (size_t)m * n_slots + slot;
-    e.am_v1[at] = -INFINITY;
-    e.am_i1[at] = 0x7fffffff;
-    e.am_v2[at] = -INFINITY;
-  }
-}
-
-JF_DEV void am_merge(float& b1, int& bi, float& b2, float o1, int oi, float o2) {
-  if (better(o1, oi, b1, bi)) { b2 = fmaxf(b1, o2); b1 = o1; bi = oi; }
-  else { b2 = fmaxf(b2, o1); }
-}
-
-// Last CTA of a token tile: reduce the slots of rows m0..m0+BN-1. Warp w takes rows two at a
-// time, lane l the slots l, l+32, ...; each round issues all loads of 2 rows x 4 slots per lane
-// before the first merge. The merge is associative and commutative, so the result does
-// not depend on which CTA folded which tile.
-constexpr int kAmSlotLoads = 4;  // slots per lane in flight per round
-JF_DEV void argmax_finish(const GemmEpi& e, int m0, int BN, int n_slots, int tid) {
-  const int warp = tid >> 5, lane = tid & 31;
-  for (int r0 = warp * 2; r0 < BN; r0 += 8) {
-    float b1[2] = {-INFINITY, -INFINITY}, b2[2] = {-INFINITY, -INFINITY};
-    int bi[2] = {0x7fffffff, 0x7fffffff};
-    for (int s0 = 0; s0 < n_slots; s0 += 32 * kAmSlotLoads) {
-      float v1[2][kAmSlotLoads], v2[2][kAmSlotLoads];
-      int i1[2][kAmSlotLoads];
-#pragma unroll
-      for (int q = 0; q < 2; ++q) {
-        const int m = m0 + r0 + q;
-#pragma unroll
-        for (int k = 0; k < kAmSlotLoads; ++k) {
-          const int s = s0 + lane + 32 * k;
-          const bool ok = (r0 + q < BN) && m < e.M && s < n_slots;
-          const size_t at = (size_t)(ok ? m : 0) * n_slots + (ok ? s : 0);
-          v1[q][k] = ok ? __ldcg(e.am_v1 + at) : -INFINITY;
-          i1[q][k] = ok ? __ldcg(e.am_i1 + at) : 0x7fffffff;
-          v2[q][k] = ok ? __ldcg(e.am_v2 + at) : -INFINITY;
-        }
-      }
-#pragma unroll
-      for (int q = 0; q < 2; ++q)
-#pragma unroll
-        for (int k = 0; k < kAmSlotLoads; ++k) am_merge(b1[q], bi[q], b2[q], v1[q][k], i1[q][k], v2[q][k]);
-    }
-#pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      const int m = m0 + r0 + q;
-      float b1q = b1[q], b2q = b2[q];
-      int biq = bi[q];
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        const float o1 = __shfl_xor_sync(0xffffffffu, b1q, o);
-        const int oi = __shfl_xor_sync(0xffffffffu, biq, o);
-        const float o2 = __shfl_xor_sync(0xffffffffu, b2q, o);
-        am_merge(b1q, biq, b2q, o1, oi, o2);
-      }
-      if (lane == 0 && r0 + q < BN && m < e.M) {
-        e.am_out[m] = biq;
-        if (e.top2_out) { e.top2_out[2 * m] = b1q; e.top2_out[2 * m + 1] = b2q; }
-      }
+      // fold this tile into the CTA's running entry of row m; the same thread owns the row's entry for
+      // every tile of the CTA, so program order orders the updates
+      const size_t at = (size_t)m * am.stride;
+      am_merge(b1, bi, b2, am.k1[at], am.idx[at], am.k2[at]);
+      am.k1[at] = b1;
+      am.idx[at] = bi;
+      am.k2[at] = b2;
     }
   }
 }
 
 template <typename T, int BN, int EPI, typename Get>
 JF_DEV void finish_tile_epi(const GemmParams& p, Get get, float* xs, int* sflag, int n_tile, int split, int m_tile,
-                            int tid, int slot, int n_slots, int n0, int m0, int tile_lin, int nchunks);
+                            int tid, const AmEntries& am, int n0, int m0, int tile_lin, int nchunks);
 
 // Shared tail of both mainloops, run by the 128 epilogue threads (tid 0..127): the partial tile
-// for EPI_PARTIAL; otherwise ticketing for split-K and argmax, then the epilogue. get(c0, v) fills
-// this thread's 16 accumulator values of columns c0..c0+15. slot of n_slots: this CTA's argmax slots.
+// for EPI_PARTIAL; otherwise ticketing for split-K, then the epilogue. get(c0, v) fills
+// this thread's 16 accumulator values of columns c0..c0+15. am: this CTA's argmax entries.
 template <typename T, int BN, int EPI, typename Get>
 JF_DEV void finish_tile(const GemmParams& p, Get get, float* xs, int* sflag, int n_tile, int split, int m_tile,
-                        int tid, int slot, int n_slots) {
+                        int tid, const AmEntries& am) {
   const int n0 = n_tile * kTileN, m0 = m_tile * BN;
   const int tile_lin = n_tile * p.m_tiles + m_tile;
   int ncols = p.M - m0;
@@ -286,19 +311,19 @@ JF_DEV void finish_tile(const GemmParams& p, Get get, float* xs, int* sflag, int
       for (int j = 0; j < 16; ++j) mine[(c * 16 + j) * kTileN + tid] = v[j];
     }
   } else {
-    finish_tile_epi<T, BN, EPI>(p, get, xs, sflag, n_tile, split, m_tile, tid, slot, n_slots, n0, m0, tile_lin,
+    finish_tile_epi<T, BN, EPI>(p, get, xs, sflag, n_tile, split, m_tile, tid, am, n0, m0, tile_lin,
                                   nchunks);
   }
 }
 
 template <typename T, int BN, int EPI, typename Get>
 JF_DEV void finish_tile_epi(const GemmParams& p, Get get, float* xs, int* sflag, int n_tile, int split, int m_tile,
-                            int tid, int slot, int n_slots, int n0, int m0, int tile_lin, int nchunks) {
+                            int tid, const AmEntries& am, int n0, int m0, int tile_lin, int nchunks) {
   if (p.k_splits == 1) {
     for (int c = 0; c < nchunks; ++c) {
       float v[16];
       get(c * 16, v);
-      epilogue_chunk<T, EPI>(p.epi, v, tid, n0, m0, c * 16, xs, n_tile, slot, n_slots);
+      epilogue_chunk<T, EPI>(p.epi, v, tid, n0, m0, c * 16, xs, n_tile, am);
     }
   } else {
     float* mine = p.ws + ((size_t)tile_lin * p.k_splits + split) * (size_t)BN * kTileN;
@@ -339,25 +364,9 @@ JF_DEV void finish_tile_epi(const GemmParams& p, Get get, float* xs, int* sflag,
           for (int j = 0; j < 16; ++j) v[j] += part[s][j];
         }
       }
-      epilogue_chunk<T, EPI>(p.epi, v, tid, n0, m0, c * 16, xs, n_tile, slot, n_slots);
+      epilogue_chunk<T, EPI>(p.epi, v, tid, n0, m0, c * 16, xs, n_tile, am);
     }
     if (tid == 0) p.tile_counter[tile_lin] = 0;
-  }
-  if constexpr (EPI == EPI_ARGMAX) {
-    __threadfence();
-    epi_sync();
-    if (tid == 0) {
-      const int t = atomicAdd(p.epi.am_counter + m_tile, 1);
-      *sflag = (t == p.n_tiles - 1);
-    }
-    epi_sync();
-    const bool last = *sflag != 0;
-    epi_sync();
-    if (last) {
-      __threadfence();
-      argmax_finish(p.epi, m0, BN, n_slots, tid);
-      if (tid == 0) p.epi.am_counter[m_tile] = 0;
-    }
   }
 }
 
@@ -621,8 +630,12 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     // epilogue warps 0-3
     pdl_wait();
     JF_TL_WAITED();
+    uint32_t* words = reinterpret_cast<uint32_t*>(xs);
+    const bool table = p.M <= kAmTableRows;
+    AmEntries am = {};
     if constexpr (EPI == EPI_ARGMAX) {
-      argmax_init_slots(p.epi, 0, p.M, blockIdx.x, gridDim.x, tid, 128);
+      am = table ? am_shared(words) : am_global(p.epi, words, blockIdx.x, gridDim.x);
+      am_clear(am, 0, p.M, tid, 128);
       epi_sync();
     }
     const uint32_t tmem = *tmem_slot;
@@ -640,12 +653,23 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
       auto get = [&](int c0, float (&v)[16]) { tmem_ld16(dacc + (uint32_t)c0, v); };
       const int n_tile = w.n_tile * kCtas + rank;
       if (n_tile < p.n_tiles)  // (the last pair's second tile may not exist)
-        finish_tile<bf16, BN, EPI>(p, get, xs, sflag, n_tile, w.split, w.m_tile, tid, blockIdx.x, gridDim.x);
+        finish_tile<bf16, BN, EPI>(p, get, xs, sflag, n_tile, w.split, w.m_tile, tid, am);
       tc_fence_before();
       epi_sync();
       if (tid == 0) {
         if constexpr (PAIR) mbar_arrive_cluster(map_to_rank(tempty0 + 8 * acc, 0));
         else mbar_arrive(tempty0 + 8 * acc);
+      }
+    }
+    if constexpr (EPI == EPI_ARGMAX) {
+      if (table) {
+        epi_sync();
+        const AmEntries out = am_global(p.epi, words, blockIdx.x, gridDim.x);
+        for (int m = tid; m < p.M; m += 128) {
+          out.k1[m * out.stride] = am.k1[m];
+          out.idx[m * out.stride] = am.idx[m];
+          out.k2[m * out.stride] = am.k2[m];
+        }
       }
     }
   }
@@ -770,11 +794,13 @@ __global__ void __launch_bounds__(F32_THREADS) k_gemm_f32(const float* __restric
         for (int j = 0; j < 16; ++j) v[j] += ld_cluster_f32(part + (c0 + j) * kTileN + row, (uint32_t)r);
       }
     };
+    AmEntries am = {};
     if constexpr (EPI == EPI_ARGMAX) {
-      argmax_init_slots(p.epi, m0, m0 + BN, n_tile, p.n_tiles, tid, 128);
+      am = am_global(p.epi, reinterpret_cast<uint32_t*>(xs), n_tile, p.n_tiles);
+      am_clear(am, m0, m0 + BN < p.M ? m0 + BN : p.M, tid, 128);
       epi_sync();
     }
-    finish_tile<float, BN, EPI>(p, get, xs, &sflag, n_tile, 0, blockIdx.z, tid, n_tile, p.n_tiles);
+    finish_tile<float, BN, EPI>(p, get, xs, &sflag, n_tile, 0, blockIdx.z, tid, am);
   }
   if (n_splits > 1) cluster_sync();  // the other CTAs keep their partial tiles until rank 0 has read them
 }
@@ -799,7 +825,9 @@ cudaError_t launch_tc_epi(const CUtensorMap& tmA, const CUtensorMap& tmB, const 
   at[1].val.clusterDim.z = 1;
   cfg.attrs = at;
   cfg.numAttrs = PAIR ? 2 : 1;
-  return cudaLaunchKernelEx(&cfg, k_gemm_tc<BN, EPI, PAIR>, tmA, tmB, p);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, k_gemm_tc<BN, EPI, PAIR>, tmA, tmB, p);
+  if (EPI != EPI_ARGMAX || e != cudaSuccess) return e;
+  return launch_argmax_finish(p.epi, p.M, (int)cfg.gridDim.x, st);
 }
 
 template <int BN, bool PAIR = false>
@@ -941,7 +969,9 @@ static cudaError_t launch_f32_epi(const float* W, const float* X, GemmParams p, 
   at[1].val.clusterDim.z = 1;
   cfg.attrs = at;
   cfg.numAttrs = splits > 1 ? 2 : 1;
-  return cudaLaunchKernelEx(&cfg, k_gemm_f32<BN, EPI>, W, X, p, splits, vec);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, k_gemm_f32<BN, EPI>, W, X, p, splits, vec);
+  if (EPI != EPI_ARGMAX || e != cudaSuccess) return e;
+  return launch_argmax_finish(p.epi, p.M, p.n_tiles, st);
 }
 
 template <int BN>

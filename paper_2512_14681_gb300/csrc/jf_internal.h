@@ -92,12 +92,11 @@ struct GemmEpi {
   // EPI_SWIGLU: tile t holds features 64t..64t+63 as row pairs (gate 64t+i at 2i, up at 2i+1); act[m][64t + i]
   void* act;
   int ld_act;
-  // EPI_ARGMAX: per (row, CTA) running (v1, i1, v2) slot, one ticket per token tile; the CTA that
-  // completes a token tile folds the slots into the final argmax / top-2
+  // EPI_ARGMAX: per (row, CTA) a slot of the best value, its index and the runner-up (values as
+  // order-preserving keys); a second kernel merges them into the final argmax / top-2
   float* am_v1;
   int* am_i1;
   float* am_v2;
-  int* am_counter;
   int* am_out;
   float* top2_out;
 };

@@ -125,7 +125,7 @@ struct Offsets {
   size_t k_pages, v_pages, page_table, seq_len, commit;
   size_t k_inf, v_inf, x, h, q, att, act;
   size_t tok, pos, gpred, top2, chains, n_chains, attn_xchg;
-  size_t gemm_ws, gemm_counter, am_v1, am_i1, am_v2, am_counter;
+  size_t gemm_ws, gemm_counter, am_v1, am_i1, am_v2;
   size_t logits, err, traj_count;
   size_t gen_state, gen_out, gen_truth, gen_log, gen_q0, gen_plast, gen_prompt, gen_seqp, res, step_blocks, step_res,
       committed;
@@ -249,7 +249,6 @@ Offsets plan_offsets(const Dims& D) {
   o.am_v1 = p.take((size_t)D.R * std::max(D.n_vtiles, kMaxGemmGrid) * 4);  // [row][CTA slot]
   o.am_i1 = p.take((size_t)D.R * std::max(D.n_vtiles, kMaxGemmGrid) * 4);  // [row][CTA slot]
   o.am_v2 = p.take((size_t)D.R * std::max(D.n_vtiles, kMaxGemmGrid) * 4);  // [row][CTA slot]
-  o.am_counter = p.take((size_t)max_mt * 4);
   o.logits = p.take((size_t)std::max(D.logits_rows, 1) * D.V * 4, 1024);
   o.err = p.take(16);
   o.traj_count = p.take(16);
@@ -326,7 +325,7 @@ struct jf_ctx {
   float* gemm_ws;
   int* gemm_counter;
   float *am_v1, *am_v2;
-  int *am_i1, *am_counter;
+  int* am_i1;
   float* logits;
   int* err;
   int *gen_state, *gen_out, *gen_truth, *gen_log, *gen_q0, *gen_plast, *gen_prompt, *gen_seqp, *traj_count;
@@ -590,12 +589,12 @@ cudaError_t enqueue_forward(jf_ctx* c, int M, LmMode lm) {
   GemmEpi el = {};
   if (lm != LM_LOGITS) {
     el.kind = EPI_ARGMAX;
-    el.am_v1 = c->am_v1; el.am_i1 = c->am_i1; el.am_v2 = c->am_v2; el.am_counter = c->am_counter;
+    el.am_v1 = c->am_v1; el.am_i1 = c->am_i1; el.am_v2 = c->am_v2;
     el.am_out = c->gpred; el.top2_out = c->top2;
   } else {
     el.kind = EPI_STORE; el.y = c->logits; el.ldy = D.V;
   }
-  c->launches += 1 + (qkv_partial ? 8LL : 7LL) * D.L + 2;
+  c->launches += 1 + (qkv_partial ? 8LL : 7LL) * D.L + (lm != LM_LOGITS ? 3 : 2);
   return gemm(c, c->tm_lm, c->w_lm, c->h, D.V, D.d, lm_rows, el, PC_LMHEAD);
 }
 
@@ -1076,7 +1075,6 @@ jf_status jf_create(const jf_model_config* model, const jf_runtime_config* rt, j
   c->am_v1 = at<float>(c, O.am_v1);
   c->am_i1 = at<int>(c, O.am_i1);
   c->am_v2 = at<float>(c, O.am_v2);
-  c->am_counter = at<int>(c, O.am_counter);
   c->logits = at<float>(c, O.logits);
   c->err = at<int>(c, O.err);
   c->gen_state = at<int>(c, O.gen_state);
@@ -1105,7 +1103,6 @@ jf_status jf_create(const jf_model_config* model, const jf_runtime_config* rt, j
   zero(O.seq_len, (size_t)D.S * 4);
   zero(O.commit, (size_t)D.S * sizeof(CommitInfo));
   zero(O.gemm_counter, (O.am_v1 - O.gemm_counter));
-  zero(O.am_counter, (size_t)(cdiv(D.R, 16) + 1) * 4);
   zero(O.err, 16);
   zero(O.n_chains, 16);
   zero(O.x, (size_t)D.R * D.d * 4);

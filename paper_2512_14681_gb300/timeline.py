@@ -26,7 +26,7 @@ REC = np.dtype([("kid", "<u4"), ("blk", "<u4"), ("smid", "<u4"), ("pad", "<u4"),
                 ("t0", "<u8"), ("t1", "<u8"), ("t2", "<u8")])
 NAMES = {1: "rmsnorm", 2: "rmsnorm+partials", 3: "qkv finish", 5: "attention", 10: "gemm store", 11: "gemm resid",
          12: "gemm qkv", 13: "gate/up (swiglu)", 14: "lm head (argmax)", 15: "gemm partials", 20: "embedding",
-         21: "acceptance", 22: "kv commit"}
+         21: "acceptance", 22: "kv commit", 23: "argmax finish"}
 
 
 def launches(rec):
