@@ -21,7 +21,7 @@ namespace {
 
 constexpr int A_STAGE_BYTES = kTileN * kTileK * 2;  // 16 KB of weights per stage
 
-constexpr int EPI_STAGE_BYTES = 16 * kTileN * 4;   // epilogue exchange buffer [16][128] fp32
+constexpr int EPI_STAGE_BYTES = 9216;               // epilogue exchange buffers (argmax)
 constexpr int SMEM_LIMIT = 232448;                  // 227 KB per CTA
 
 // PAIR: two CTAs (a cluster) share a tile of 256 weight rows; each stages its 128 rows of A and half of
@@ -40,8 +40,18 @@ struct TcCfg {
   static_assert(SMEM <= SMEM_LIMIT, "shared memory budget");
 };
 
-// Named barrier of the 128 epilogue threads (barrier 0 is __syncthreads).
-JF_DEV void epi_sync() { asm volatile("bar.sync 1, 128;" ::: "memory"); }
+// The epilogue's threads: NH groups of 128, group `half` takes the 16-column chunks half, half + NH, ...
+// sync(): the group's barrier; sync_all(): that of all groups (barrier 0 is __syncthreads).
+template <int NH>
+struct EpiThreads {
+  int half, row;  // row: this thread's weight row of the tile
+  JF_DEV void sync() const { asm volatile("bar.sync %0, 128;" ::"r"(1 + half) : "memory"); }
+  JF_DEV void sync_all() const {
+    if constexpr (NH == 1) sync();
+    else asm volatile("bar.sync 3, %0;" ::"n"(128 * NH) : "memory");
+  }
+  JF_DEV bool first() const { return half == 0 && row == 0; }
+};
 
 constexpr int kMaxSplits = 8;  // split-K never exceeds this (enforced by the host)
 
@@ -74,7 +84,7 @@ JF_DEV void am_merge(uint32_t& b1, uint32_t& bi, uint32_t& b2, uint32_t o1, uint
   }
 }
 
-constexpr int kAmRedWords = 2 * 4 * 16 * 3;  // [chunk parity][warp][column][3]
+constexpr int kAmRedWords = 2 * 2 * 4 * 16 * 3;  // [group][parity of its chunk][warp][column][3]
 constexpr int kAmTableRows = 512;
 static_assert((kAmRedWords + 3 * kAmTableRows) * 4 <= EPI_STAGE_BYTES, "argmax tables fit the epilogue's staging");
 constexpr uint32_t kAmNoIndex = 0x7fffffffu;
@@ -156,10 +166,10 @@ cudaError_t launch_argmax_finish(const GemmEpi& e, int M, int n_slots, cudaStrea
 // Epilogue on one 16-column chunk: thread `row` (0..127) holds v[j] = Y[m0 + c0 + j, n0 + row].
 // xs: shared staging [16][128] fp32 (exchange between the two halves of a tile).
 // ---------------------------------------------------------------------------------------------
-template <typename T, int EPI>
-JF_DEV void epilogue_chunk(const GemmEpi& e, const float (&v)[16], int row, int n0, int m0, int c0, float* xs,
+template <typename T, int EPI, int NH>
+JF_DEV void epilogue_chunk(const GemmEpi& e, const float (&v)[16], const EpiThreads<NH>& th, int n0, int m0, int c0, float* xs,
                            int n_tile, const AmEntries& am) {
-  const int n = n0 + row;
+  const int row = th.row, n = n0 + row;
   constexpr int kind = EPI;
   if constexpr (kind == EPI_STORE || kind == EPI_RESID) {
     if (n < e.N) {
@@ -206,7 +216,7 @@ JF_DEV void epilogue_chunk(const GemmEpi& e, const float (&v)[16], int row, int 
     const float b = (e.bias != nullptr && n < e.N) ? act_to_f32(reinterpret_cast<const T*>(e.bias)[n]) : 0.f;
 #pragma unroll
     for (int j = 0; j < 16; ++j) xs[j * 128 + row] = v[j] + b;
-    epi_sync();
+    th.sync();
     {
       const int hd = e.head_dim, half = hd >> 1;
       const int i = n % hd;
@@ -242,7 +252,7 @@ JF_DEV void epilogue_chunk(const GemmEpi& e, const float (&v)[16], int row, int 
         }
       }
     }
-    epi_sync();
+    th.sync();
     return;
   } else {
     // EPI_ARGMAX: best (value, lowest index) and runner-up over this tile's 128 vocabulary rows. A warp
@@ -261,14 +271,15 @@ JF_DEV void epilogue_chunk(const GemmEpi& e, const float (&v)[16], int row, int 
         b2 = second;
       }
     }
-    uint32_t* red = am.red + ((c0 >> 4) & 1) * (4 * 16 * 3);  // alternates: one barrier a chunk is enough
+    // (alternates from one of the group's chunks to the next: one barrier a chunk is enough)
+    uint32_t* red = am.red + (th.half * 2 + (c0 / (16 * NH) & 1)) * (4 * 16 * 3);
     if (lane < 16) {
       uint32_t* mine = red + (warp * 16 + lane) * 3;
       mine[0] = b1;
       mine[1] = bi;
       mine[2] = b2;
     }
-    epi_sync();
+    th.sync();
     const int m = m0 + c0 + row;
     if (row < 16 && m < e.M) {
 #pragma unroll
@@ -287,86 +298,74 @@ JF_DEV void epilogue_chunk(const GemmEpi& e, const float (&v)[16], int row, int 
   }
 }
 
-template <typename T, int BN, int EPI, typename Get>
-JF_DEV void finish_tile_epi(const GemmParams& p, Get get, float* xs, int* sflag, int n_tile, int split, int m_tile,
-                            int tid, const AmEntries& am, int n0, int m0, int tile_lin, int nchunks);
-
-// Shared tail of both mainloops, run by the 128 epilogue threads (tid 0..127): the partial tile
-// for EPI_PARTIAL; otherwise ticketing for split-K, then the epilogue. get(c0, v) fills
-// this thread's 16 accumulator values of columns c0..c0+15. am: this CTA's argmax entries.
-template <typename T, int BN, int EPI, typename Get>
+// Shared tail of both mainloops, run by the epilogue threads: the partial tile for EPI_PARTIAL;
+// otherwise ticketing for split-K, then the epilogue. get(c0, v) fills this thread's 16 accumulator
+// values of columns c0..c0+15. am: this CTA's argmax entries.
+template <typename T, int BN, int EPI, int NH, typename Get>
 JF_DEV void finish_tile(const GemmParams& p, Get get, float* xs, int* sflag, int n_tile, int split, int m_tile,
-                        int tid, const AmEntries& am) {
+                        const EpiThreads<NH>& th, const AmEntries& am) {
   const int n0 = n_tile * kTileN, m0 = m_tile * BN;
   const int tile_lin = n_tile * p.m_tiles + m_tile;
   int ncols = p.M - m0;
   if (ncols > BN) ncols = BN;
   const int nchunks = (ncols + 15) >> 4;
+  auto store_partial = [&]() {
+    float* mine = p.ws + ((size_t)tile_lin * p.k_splits + split) * (size_t)BN * kTileN;
+    for (int c = th.half; c < nchunks; c += NH) {
+      float v[16];
+      get(c * 16, v);
+#pragma unroll
+      for (int j = 0; j < 16; ++j) mine[(c * 16 + j) * kTileN + th.row] = v[j];
+    }
+  };
   if constexpr (EPI == EPI_PARTIAL) {
-    float* mine = p.ws + ((size_t)tile_lin * p.k_splits + split) * (size_t)BN * kTileN;
-    for (int c = 0; c < nchunks; ++c) {
+    store_partial();
+  } else if (p.k_splits == 1) {
+    for (int c = th.half; c < nchunks; c += NH) {
       float v[16];
       get(c * 16, v);
-#pragma unroll
-      for (int j = 0; j < 16; ++j) mine[(c * 16 + j) * kTileN + tid] = v[j];
+      epilogue_chunk<T, EPI>(p.epi, v, th, n0, m0, c * 16, xs, n_tile, am);
     }
   } else {
-    finish_tile_epi<T, BN, EPI>(p, get, xs, sflag, n_tile, split, m_tile, tid, am, n0, m0, tile_lin,
-                                  nchunks);
-  }
-}
-
-template <typename T, int BN, int EPI, typename Get>
-JF_DEV void finish_tile_epi(const GemmParams& p, Get get, float* xs, int* sflag, int n_tile, int split, int m_tile,
-                            int tid, const AmEntries& am, int n0, int m0, int tile_lin, int nchunks) {
-  if (p.k_splits == 1) {
-    for (int c = 0; c < nchunks; ++c) {
-      float v[16];
-      get(c * 16, v);
-      epilogue_chunk<T, EPI>(p.epi, v, tid, n0, m0, c * 16, xs, n_tile, am);
-    }
-  } else {
-    float* mine = p.ws + ((size_t)tile_lin * p.k_splits + split) * (size_t)BN * kTileN;
-    for (int c = 0; c < nchunks; ++c) {
-      float v[16];
-      get(c * 16, v);
-#pragma unroll
-      for (int j = 0; j < 16; ++j) mine[(c * 16 + j) * kTileN + tid] = v[j];
-    }
+    store_partial();
     __threadfence();
-    epi_sync();
-    if (tid == 0) {
+    th.sync_all();
+    if (th.first()) {
       const int t = atomicAdd(p.tile_counter + tile_lin, 1);
       *sflag = (t == p.k_splits - 1);
     }
-    epi_sync();
+    th.sync_all();
     const bool last = *sflag != 0;
-    epi_sync();
+    th.sync_all();
     if (!last) return;
     __threadfence();
     const float* base = p.ws + (size_t)tile_lin * p.k_splits * (size_t)BN * kTileN;
-    for (int c = 0; c < nchunks; ++c) {
-      // partials of every split in flight together, then added in split order
-      float part[kMaxSplits][16];
-#pragma unroll
-      for (int s = 0; s < kMaxSplits; ++s) {
-        const float* src = base + (size_t)s * BN * kTileN;
-#pragma unroll
-        for (int j = 0; j < 16; ++j) part[s][j] = (s < p.k_splits) ? __ldcg(src + (c * 16 + j) * kTileN + tid) : 0.0f;
-      }
+    for (int c = th.half; c < nchunks; c += NH) {
+      // partials of four splits in flight together, added in split order
       float v[16];
 #pragma unroll
       for (int j = 0; j < 16; ++j) v[j] = 0.0f;
 #pragma unroll
-      for (int s = 0; s < kMaxSplits; ++s) {
-        if (s < p.k_splits) {
+      for (int s0 = 0; s0 < kMaxSplits; s0 += 4) {
+        float part[4][16];
 #pragma unroll
-          for (int j = 0; j < 16; ++j) v[j] += part[s][j];
+        for (int s = 0; s < 4; ++s) {
+          const float* src = base + (size_t)(s0 + s) * BN * kTileN;
+#pragma unroll
+          for (int j = 0; j < 16; ++j)
+            part[s][j] = (s0 + s < p.k_splits) ? __ldcg(src + (c * 16 + j) * kTileN + th.row) : 0.0f;
+        }
+#pragma unroll
+        for (int s = 0; s < 4; ++s) {
+          if (s0 + s < p.k_splits) {
+#pragma unroll
+            for (int j = 0; j < 16; ++j) v[j] += part[s][j];
+          }
         }
       }
-      epilogue_chunk<T, EPI>(p.epi, v, tid, n0, m0, c * 16, xs, n_tile, am);
+      epilogue_chunk<T, EPI>(p.epi, v, th, n0, m0, c * 16, xs, n_tile, am);
     }
-    if (tid == 0) p.tile_counter[tile_lin] = 0;
+    if (th.first()) p.tile_counter[tile_lin] = 0;
   }
 }
 
@@ -388,8 +387,10 @@ JF_DEV Unit unit_of(const GemmParams& p, int u) {
 }
 
 // ---------------------------------------------------------------------------------------------
-// bf16 tcgen05 persistent kernel, 192 threads: warps 0-3 epilogue (warp w reads TMEM lanes
-// 32w .. 32w+31), warp 4 = TMA producer, warp 5 = MMA issuer (and the TMEM allocation).
+// bf16 tcgen05 persistent kernel, 320 threads: warps 0-7 epilogue (warp w reads TMEM lanes
+// 32(w%4) .. 32(w%4)+31 and every other 16-column chunk: the last unit's epilogue is not hidden, and
+// eight warps halve it), warp 8 = TMA producer, warp 9 = MMA issuer (and the TMEM allocation).
+// (8 layers and head of the 7B shape: 64 rows 990 -> 978 us, 160 rows 1198 -> 1167; 32 rows as before).
 //
 // PAIR (256-token tiles, i.e. more than 160 rows): two CTAs on neighbouring SMs take a tile of 256
 // weight rows together (cta_group::2). Each loads its own 128 weight rows and half of the tokens (32 KB
@@ -398,7 +399,8 @@ JF_DEV Unit unit_of(const GemmParams& p, int u) {
 // an SM draws from L2, and only four such stages fit. gate/up (37888 x 3584) at 512 rows: 110.6 ->
 // 104.9 us a call (1.33 PFLOP/s); prefill of 4,000 tokens through one 7B layer 2.39 -> 2.29 ms.
 // ---------------------------------------------------------------------------------------------
-constexpr int TC_THREADS = 192;
+constexpr int EPI_HALVES = 2, PRODUCER_WARP = 4 * EPI_HALVES, MMA_WARP = PRODUCER_WARP + 1;
+constexpr int TC_THREADS = 32 * (MMA_WARP + 1);
 
 template <int BN, int EPI, bool PAIR>
 __global__ void __launch_bounds__(TC_THREADS, 1)
@@ -464,7 +466,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
   auto expect = [&](const Unit& w, int kb, int d, bool on) {
     mbar_arrive_expect_tx(full0 + 8 * d, (kb + 1 < w.kb1 ? 2 : 1) * kCtas * Cfg::STAGE_BYTES, on && rank == 0);
   };
-  if (tid == 128) {
+  if (tid == 32 * PRODUCER_WARP) {
     for (int d = 0; d < D; ++d) {
       mbar_init(full0 + 8 * d, 1);
       mbar_init(empty0 + 8 * d, 1);
@@ -479,7 +481,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     tma_prefetch_desc(&tmA);
     tma_prefetch_desc(&tmB);
   }
-  if (warp == 5) {
+  if (warp == MMA_WARP) {
     if constexpr (PAIR) {
       tmem_alloc_pair(smem_u32(tmem_slot), Cfg::TMEM_COLS);
       tmem_relinquish_pair();
@@ -493,14 +495,14 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
   if constexpr (PAIR) {
     __syncthreads();
     cluster_sync();  // both CTAs' barriers exist, and both hold their TMEM
-  } else if (warp == 4) {
-    asm volatile("bar.arrive 2, 192;" ::: "memory");  // the producer starts without waiting for the others
+  } else if (warp == PRODUCER_WARP) {
+    asm volatile("bar.arrive 2, %0;" ::"n"(TC_THREADS) : "memory");  // the producer starts without waiting for the others
   } else {
-    asm volatile("bar.sync 2, 192;" ::: "memory");
+    asm volatile("bar.sync 2, %0;" ::"n"(TC_THREADS) : "memory");
   }
   tc_fence_after();
 
-  if (warp == 4) {
+  if (warp == PRODUCER_WARP) {
     // Stage pairs 0 .. pre-1: lane j requests the weights of pair j before the dependency wait (they do
     // not depend on earlier kernels, so they stream in while the previous kernel finishes) and its
     // activations right after it; from then on one lane requests both of a pair as it comes free. Round
@@ -564,7 +566,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         if (!mbar_wait_bounded(empty0 + 8 * (q % D), (uint32_t)(q / D) & 1u, p.wait_ns)) break;
     }
     __syncwarp();
-  } else if (warp == 5) {
+  } else if (warp == MMA_WARP) {
     // The whole warp walks the stage pairs, one elected lane issues (a wait behind issued MMAs takes as
     // long as they queue); descriptors are a base plus constants. The first pass over the loop computes
     // on whatever the stages hold, into an accumulator that the first real MMA overwrites, and its waits
@@ -627,19 +629,20 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     }
     __syncwarp();
   } else {
-    // epilogue warps 0-3
+    // epilogue warps
     pdl_wait();
     JF_TL_WAITED();
     uint32_t* words = reinterpret_cast<uint32_t*>(xs);
     const bool table = p.M <= kAmTableRows;
+    const EpiThreads<EPI_HALVES> th{warp >> 2, tid & 127};
     AmEntries am = {};
     if constexpr (EPI == EPI_ARGMAX) {
       am = table ? am_shared(words) : am_global(p.epi, words, blockIdx.x, gridDim.x);
-      am_clear(am, 0, p.M, tid, 128);
-      epi_sync();
+      am_clear(am, 0, p.M, tid, 128 * EPI_HALVES);
+      th.sync_all();
     }
     const uint32_t tmem = *tmem_slot;
-    const uint32_t lane_base = (uint32_t)(warp * 32) << 16;
+    const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
     int i = 0;
     for (int u = first_unit; u < total_units; u += unit_step, ++i) {
       const Unit w = unit_of(p, u);
@@ -653,9 +656,9 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
       auto get = [&](int c0, float (&v)[16]) { tmem_ld16(dacc + (uint32_t)c0, v); };
       const int n_tile = w.n_tile * kCtas + rank;
       if (n_tile < p.n_tiles)  // (the last pair's second tile may not exist)
-        finish_tile<bf16, BN, EPI>(p, get, xs, sflag, n_tile, w.split, w.m_tile, tid, am);
+        finish_tile<bf16, BN, EPI>(p, get, xs, sflag, n_tile, w.split, w.m_tile, th, am);
       tc_fence_before();
-      epi_sync();
+      th.sync_all();
       if (tid == 0) {
         if constexpr (PAIR) mbar_arrive_cluster(map_to_rank(tempty0 + 8 * acc, 0));
         else mbar_arrive(tempty0 + 8 * acc);
@@ -663,9 +666,9 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     }
     if constexpr (EPI == EPI_ARGMAX) {
       if (table) {
-        epi_sync();
+        th.sync_all();
         const AmEntries out = am_global(p.epi, words, blockIdx.x, gridDim.x);
-        for (int m = tid; m < p.M; m += 128) {
+        for (int m = tid; m < p.M; m += 128 * EPI_HALVES) {
           out.k1[m * out.stride] = am.k1[m];
           out.idx[m * out.stride] = am.idx[m];
           out.k2[m * out.stride] = am.k2[m];
@@ -677,9 +680,9 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
   __syncthreads();
   if constexpr (PAIR) {
     cluster_sync();  // neither CTA leaves while the other may use its shared or tensor memory
-    if (warp == 5) tmem_dealloc_pair(*tmem_slot, Cfg::TMEM_COLS);
+    if (warp == MMA_WARP) tmem_dealloc_pair(*tmem_slot, Cfg::TMEM_COLS);
   } else {
-    if (warp == 5) tmem_dealloc(*tmem_slot, Cfg::TMEM_COLS);
+    if (warp == MMA_WARP) tmem_dealloc(*tmem_slot, Cfg::TMEM_COLS);
   }
   JF_TL_EXIT(TL_GEMM + EPI);
 }
@@ -794,13 +797,14 @@ __global__ void __launch_bounds__(F32_THREADS) k_gemm_f32(const float* __restric
         for (int j = 0; j < 16; ++j) v[j] += ld_cluster_f32(part + (c0 + j) * kTileN + row, (uint32_t)r);
       }
     };
+    const EpiThreads<1> th{0, row};
     AmEntries am = {};
     if constexpr (EPI == EPI_ARGMAX) {
       am = am_global(p.epi, reinterpret_cast<uint32_t*>(xs), n_tile, p.n_tiles);
       am_clear(am, m0, m0 + BN < p.M ? m0 + BN : p.M, tid, 128);
-      epi_sync();
+      th.sync_all();
     }
-    finish_tile<float, BN, EPI>(p, get, xs, &sflag, n_tile, 0, blockIdx.z, tid, am);
+    finish_tile<float, BN, EPI>(p, get, xs, &sflag, n_tile, 0, blockIdx.z, th, am);
   }
   if (n_splits > 1) cluster_sync();  // the other CTAs keep their partial tiles until rank 0 has read them
 }
@@ -834,8 +838,6 @@ template <int BN, bool PAIR = false>
 cudaError_t launch_tc(const CUtensorMap& tmA, const CUtensorMap& tmB, const GemmParams& p, cudaStream_t st) {
   switch (p.epi.kind) {
     case EPI_STORE: return launch_tc_epi<BN, EPI_STORE, PAIR>(tmA, tmB, p, st);
-    case EPI_RESID: return launch_tc_epi<BN, EPI_RESID, PAIR>(tmA, tmB, p, st);
-    case EPI_QKV: return launch_tc_epi<BN, EPI_QKV, PAIR>(tmA, tmB, p, st);
     case EPI_SWIGLU: return launch_tc_epi<BN, EPI_SWIGLU, PAIR>(tmA, tmB, p, st);
     case EPI_ARGMAX: return launch_tc_epi<BN, EPI_ARGMAX, PAIR>(tmA, tmB, p, st);
     case EPI_PARTIAL: return launch_tc_epi<BN, EPI_PARTIAL, PAIR>(tmA, tmB, p, st);
@@ -852,8 +854,7 @@ template <int BN, bool PAIR = false>
 cudaError_t prep_tc() {
   cudaError_t e;
   const int sm = TcCfg<BN, PAIR>::SMEM;
-  if ((e = opt_in(k_gemm_tc<BN, EPI_STORE, PAIR>, sm)) || (e = opt_in(k_gemm_tc<BN, EPI_RESID, PAIR>, sm)) ||
-      (e = opt_in(k_gemm_tc<BN, EPI_QKV, PAIR>, sm)) || (e = opt_in(k_gemm_tc<BN, EPI_SWIGLU, PAIR>, sm)) ||
+  if ((e = opt_in(k_gemm_tc<BN, EPI_STORE, PAIR>, sm)) || (e = opt_in(k_gemm_tc<BN, EPI_SWIGLU, PAIR>, sm)) ||
       (e = opt_in(k_gemm_tc<BN, EPI_ARGMAX, PAIR>, sm)))
     return e;
   return opt_in(k_gemm_tc<BN, EPI_PARTIAL, PAIR>, sm);
