@@ -250,6 +250,108 @@ __global__ void __launch_bounds__(NORM_THREADS) k_rmsnorm(float* __restrict__ x,
   JF_TL_EXIT(KS > 0 ? TL_NORM_ACC : TL_NORM);
 }
 
+// The same rows with 256 threads each, for launches of more rows than the GPU holds CTAs of 1024 threads
+// (one per SM: 512 rows took 10.5 us in four waves). 8 layers and head of the 7B shape: 160 rows 1151 ->
+// 1137 us, 512 rows 2072 -> 2038; up to 152 rows the one wave of 1024-thread CTAs is the faster (its CTAs
+// leave the next projection's weight prefetch room: 256-thread ones made 16 rows of the 1.5B shape 403 ->
+// 424 us). Thread t holds the
+// vectors of threads t, t + 256, t + 512 and t + 768 above, so that every sum has the same terms in the
+// same order and a row's result does not depend on the number of rows.
+constexpr int NORM_SMALL = 256;
+template <typename T, int KS>
+__global__ void __launch_bounds__(NORM_SMALL) k_rmsnorm_rows(float* __restrict__ x, const float* __restrict__ gain,
+                                                             T* __restrict__ y, int d, float eps, SplitPartials sp,
+                                                             int row0) {
+  constexpr int Q = NORM_THREADS / NORM_SMALL;
+  __shared__ float red[NORM_THREADS / 32];
+  JF_TL_ENTRY();
+  pdl_launch_dependents();
+  const int nv = d >> 2;
+  const int r = row0 + blockIdx.x;
+  float* xr = x + (size_t)r * d;
+  pdl_wait();
+  JF_TL_WAITED();
+  float4 v[Q][NORM_VEC];
+#pragma unroll
+  for (int j = 0; j < NORM_VEC; ++j) {
+#pragma unroll
+    for (int k = 0; k < Q; ++k) {
+      const int i = threadIdx.x + k * NORM_SMALL + j * NORM_THREADS;
+      v[k][j] = ldcg4_if(xr + 4 * (i < nv ? i : 0), i < nv);
+    }
+  }
+  if constexpr (KS > 0) {
+    constexpr int NB = (KS + 3) / 4;
+    const size_t stride = (size_t)sp.bn * 128;
+    const size_t tile = (size_t)sp.m_tiles * KS * sp.bn * 128;  // floats from one 128-feature tile to the next
+    const float* row = sp.ws + ((size_t)(r / sp.bn) * KS * sp.bn + (size_t)(r % sp.bn)) * 128;
+#pragma unroll
+    for (int j = 0; j < NORM_VEC; ++j) {
+      if (j * NORM_THREADS >= nv) break;
+#pragma unroll
+      for (int k0 = 0; k0 < Q; k0 += 2) {  // the partials of two vectors in flight together
+        float4 q[2][NB][4];
+#pragma unroll
+        for (int g = 0; g < 2; ++g) {
+          const int i = threadIdx.x + (k0 + g) * NORM_SMALL + j * NORM_THREADS, n = 4 * (i < nv ? i : 0);
+#pragma unroll
+          for (int b = 0; b < NB; ++b)
+            ldcg4x4(row + (size_t)(n >> 7) * tile + (n & 127) + (size_t)(4 * b) * stride, stride,
+                    i < nv ? KS - 4 * b : 0, q[g][b]);
+        }
+#pragma unroll
+        for (int g = 0; g < 2; ++g) {
+          const int k = k0 + g, i = threadIdx.x + k * NORM_SMALL + j * NORM_THREADS;
+          if (i < nv) {
+            float4 acc = q[g][0][0];
+#pragma unroll
+            for (int s = 1; s < KS; ++s) {
+              acc.x += q[g][s >> 2][s & 3].x;
+              acc.y += q[g][s >> 2][s & 3].y;
+              acc.z += q[g][s >> 2][s & 3].z;
+              acc.w += q[g][s >> 2][s & 3].w;
+            }
+            v[k][j] = make_float4(v[k][j].x + acc.x, v[k][j].y + acc.y, v[k][j].z + acc.z, v[k][j].w + acc.w);
+            store4(xr + 4 * i, v[k][j]);
+          }
+        }
+      }
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < Q; ++k) {
+    float ss = 0.f;
+#pragma unroll
+    for (int j = 0; j < NORM_VEC; ++j) {
+      ss = fmaf(v[k][j].x, v[k][j].x, ss);
+      ss = fmaf(v[k][j].y, v[k][j].y, ss);
+      ss = fmaf(v[k][j].z, v[k][j].z, ss);
+      ss = fmaf(v[k][j].w, v[k][j].w, ss);
+    }
+    ss = warp_sum(ss);
+    if ((threadIdx.x & 31) == 0) red[k * (NORM_SMALL / 32) + (threadIdx.x >> 5)] = ss;
+  }
+  __syncthreads();
+  float tot = 0.f;
+#pragma unroll
+  for (int w = 0; w < NORM_THREADS / 32; ++w) tot += red[w];
+  const float rs = 1.0f / sqrtf(tot / (float)d + eps);
+  T* yr = y + (size_t)blockIdx.x * d;
+  const float4* g4 = reinterpret_cast<const float4*>(gain);
+#pragma unroll
+  for (int j = 0; j < NORM_VEC; ++j) {
+#pragma unroll
+    for (int k = 0; k < Q; ++k) {
+      const int i = threadIdx.x + k * NORM_SMALL + j * NORM_THREADS;
+      if (i < nv) {
+        const float4 g = g4[i];
+        store4(yr + 4 * i, make_float4(v[k][j].x * rs * g.x, v[k][j].y * rs * g.y, v[k][j].z * rs * g.z, v[k][j].w * rs * g.w));
+      }
+    }
+  }
+  JF_TL_EXIT(KS > 0 ? TL_NORM_ACC : TL_NORM);
+}
+
 // Finish of the QKV projection from its split-K partials (EPI_PARTIAL, head_dim 128 = one weight
 // tile per head): for row m and head slot hs (query heads, then key heads, then value heads), add
 // the partials in split order, then the feature's bias when the model has QKV biases, rotate query and key heads by the row's position (rotate-half RoPE,
@@ -408,6 +510,8 @@ cudaError_t launch_embed(const void* E, bool is_bf16, const int* tok, float* x, 
 template <int KS>
 cudaError_t launch_rmsnorm_ks(float* x, const float* gain, bf16* y, int rows, int d, float eps,
                               const SplitPartials& sp, int row0, cudaStream_t st) {
+  if (rows > 152)
+    return launch_pdl(k_rmsnorm_rows<bf16, KS>, dim3(rows), dim3(NORM_SMALL), st, x, gain, y, d, eps, sp, row0);
   return launch_pdl(k_rmsnorm<bf16, KS>, dim3(rows), dim3(NORM_THREADS), st, x, gain, y, d, eps, sp, row0);
 }
 
