@@ -666,19 +666,21 @@ __global__ void __launch_bounds__(ATT_THREADS, 1)
   JF_TL_EXIT(TL_ATTN);
 }
 
-// fp32 path: one warp per (row, query head); keys in absolute order, 32 at a time. Latency bounds it
-// (small models, short contexts): a lane has its whole key row in flight at once (four partial dot
-// products), and the value rows are loaded eight at a time before their sums.
+// fp32 path: one CTA per (row, query head); warp w takes the absolute 32-key groups w, w + 4, ... in
+// increasing order, and the four states are folded in warp order, so a row's result does not depend on
+// the other rows. Latency bounds it (small models, short contexts): a lane has its whole key row in
+// flight at once (four partial dot products), and a group's value rows are all loaded before their sums.
+constexpr int F32_WARPS = 4;
 template <int HDT>
-__global__ void __launch_bounds__(128) k_attn_f32(const AttnParams a, int n_rows) {
+__global__ void __launch_bounds__(32 * F32_WARPS) k_attn_f32(const AttnParams a) {
   constexpr int NV = HDT / 32;  // dims per lane of the output
-  __shared__ float4 s_q[4][HDT / 4];
+  constexpr int VB = 64 / NV;   // value rows in flight (64 registers)
+  __shared__ float4 s_q[HDT / 4];
+  __shared__ float s_o[F32_WARPS][HDT], s_m[F32_WARPS], s_l[F32_WARPS];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int job = blockIdx.x * 4 + warp;
+  const int r = blockIdx.x / a.Hq, h = blockIdx.x % a.Hq;
   pdl_launch_dependents();
   pdl_wait();
-  const int r = job / a.Hq, h = job % a.Hq;
-  if (r >= n_rows) return;
   const int kvh = h / (a.Hq / a.Hkv);
   const int n_ch = *a.n_chains_dev;
   int ci = 0;
@@ -690,8 +692,8 @@ __global__ void __launch_bounds__(128) k_attn_f32(const AttnParams a, int n_rows
   const Chain ch = a.chains[ci];
   const int pos = ch.pos0 + (r - ch.row0);
   const float4* q = reinterpret_cast<const float4*>(reinterpret_cast<const float*>(a.q) + ((size_t)r * a.Hq + h) * HDT);
-  if (lane < HDT / 4) s_q[warp][lane] = q[lane];
-  __syncwarp();
+  if (threadIdx.x < HDT / 4) s_q[threadIdx.x] = q[threadIdx.x];
+  __syncthreads();
   const float* Kp = reinterpret_cast<const float*>(a.k_pages);
   const float* Vp = reinterpret_cast<const float*>(a.v_pages);
   const float* Ki = reinterpret_cast<const float*>(a.k_inf);
@@ -700,7 +702,7 @@ __global__ void __launch_bounds__(128) k_attn_f32(const AttnParams a, int n_rows
   float m = -INFINITY, l = 0.f, o[NV];
 #pragma unroll
   for (int i = 0; i < NV; ++i) o[i] = 0.f;
-  for (int kb = 0; kb <= pos; kb += 32) {
+  for (int kb = 32 * warp; kb <= pos; kb += 32 * F32_WARPS) {
     const int kp = kb + lane;
     float s = -INFINITY;
     unsigned long long v_row = 0;  // this lane's key's value row
@@ -722,7 +724,7 @@ __global__ void __launch_bounds__(128) k_attn_f32(const AttnParams a, int n_rows
         for (int i = 0; i < 16; ++i) kv[i] = kr[i0 + i];
 #pragma unroll
         for (int i = 0; i < 16; ++i) {
-          const float4 x = s_q[warp][i0 + i];
+          const float4 x = s_q[i0 + i];
           d[0] = fmaf(x.x, kv[i].x, d[0]);
           d[1] = fmaf(x.y, kv[i].y, d[1]);
           d[2] = fmaf(x.z, kv[i].z, d[2]);
@@ -740,28 +742,46 @@ __global__ void __launch_bounds__(128) k_attn_f32(const AttnParams a, int n_rows
     l = l * al + warp_sum(p);
 #pragma unroll
     for (int i = 0; i < NV; ++i) o[i] *= al;
-    for (int j0 = 0; j0 < 32 && kb + j0 <= pos; j0 += 8) {
-      float v[8][NV], pj[8];
+#pragma unroll 1
+    for (int j0 = 0; j0 < 32 && kb + j0 <= pos; j0 += VB) {
+      float v[VB][NV];
 #pragma unroll
-      for (int j = 0; j < 8; ++j) {
+      for (int j = 0; j < VB; ++j) {
         const float* vr = reinterpret_cast<const float*>(__shfl_sync(0xffffffffu, v_row, j0 + j));
-        pj[j] = __shfl_sync(0xffffffffu, p, j0 + j);
 #pragma unroll
         for (int i = 0; i < NV; ++i) v[j][i] = (kb + j0 + j <= pos) ? vr[lane + 32 * i] : 0.f;
       }
 #pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        if (kb + j0 + j > pos) break;
+      for (int j = 0; j < VB; ++j) {
+        const float pj = __shfl_sync(0xffffffffu, p, j0 + j);
+        if (kb + j0 + j <= pos) {
 #pragma unroll
-        for (int i = 0; i < NV; ++i) o[i] = fmaf(pj[j], v[j][i], o[i]);
+          for (int i = 0; i < NV; ++i) o[i] = fmaf(pj, v[j][i], o[i]);
+        }
       }
     }
     m = mn;
   }
-  float* out = reinterpret_cast<float*>(a.out) + ((size_t)r * a.Hq + h) * HDT;
-  const float il = l > 0.f ? 1.f / l : 0.f;
+  if (lane == 0) {
+    s_m[warp] = m;
+    s_l[warp] = l;
+  }
 #pragma unroll
-  for (int i = 0; i < NV; ++i) out[lane + 32 * i] = o[i] * il;
+  for (int i = 0; i < NV; ++i) s_o[warp][lane + 32 * i] = o[i];
+  __syncthreads();
+  const int dim = threadIdx.x;
+  if (dim < HDT) {
+    float M = s_m[0], L = s_l[0], acc = s_o[0][dim];  // group 0 holds key 0: never empty
+#pragma unroll
+    for (int w = 1; w < F32_WARPS; ++w) {
+      float wa, wb, mm;
+      fold_weights(M, s_m[w], wa, wb, mm);
+      M = mm;
+      L = fold_value(wa, L, wb, s_l[w]);
+      acc = fold_value(wa, acc, wb, s_o[w][dim]);
+    }
+    reinterpret_cast<float*>(a.out)[((size_t)r * a.Hq + h) * HDT + dim] = acc * (L > 0.f ? 1.f / L : 0.f);
+  }
 }
 
 }  // namespace
@@ -818,15 +838,15 @@ cudaError_t attn_prepare(int max_clusters[4]) {
 
 cudaError_t launch_attn_f32(const AttnParams& a, int n_rows, cudaStream_t st) {
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((n_rows * a.Hq + 3) / 4);
-  cfg.blockDim = dim3(128);
+  cfg.gridDim = dim3(n_rows * a.Hq);
+  cfg.blockDim = dim3(32 * F32_WARPS);
   cfg.stream = st;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, a.hd == 64 ? k_attn_f32<64> : k_attn_f32<128>, a, n_rows);
+  return cudaLaunchKernelEx(&cfg, a.hd == 64 ? k_attn_f32<64> : k_attn_f32<128>, a);
 }
 
 }  // namespace jf

@@ -792,9 +792,21 @@ __global__ void __launch_bounds__(F32_THREADS) k_gemm_f32(const float* __restric
     auto get = [&](int c0, float (&v)[16]) {
 #pragma unroll
       for (int j = 0; j < 16; ++j) v[j] = part[(c0 + j) * kTileN + row];
-      for (int r = 1; r < n_splits; ++r) {
+      for (int r0 = 1; r0 < n_splits; r0 += 4) {  // four CTAs' values in flight, added in rank order
+        float q[4][16];
 #pragma unroll
-        for (int j = 0; j < 16; ++j) v[j] += ld_cluster_f32(part + (c0 + j) * kTileN + row, (uint32_t)r);
+        for (int r = 0; r < 4; ++r) {
+#pragma unroll
+          for (int j = 0; j < 16; ++j)
+            q[r][j] = r0 + r < n_splits ? ld_cluster_f32(part + (c0 + j) * kTileN + row, (uint32_t)(r0 + r)) : 0.f;
+        }
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+          if (r0 + r < n_splits) {
+#pragma unroll
+            for (int j = 0; j < 16; ++j) v[j] += q[r][j];
+          }
+        }
       }
     };
     const EpiThreads<1> th{0, row};
