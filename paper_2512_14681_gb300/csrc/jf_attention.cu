@@ -669,7 +669,11 @@ __global__ void __launch_bounds__(ATT_THREADS, 1)
 // fp32 path: one CTA per (row, query head); warp w takes the absolute 32-key groups w, w + 4, ... in
 // increasing order, and the four states are folded in warp order, so a row's result does not depend on
 // the other rows. Latency bounds it (small models, short contexts): a lane has its whole key row in
-// flight at once (four partial dot products), and a group's value rows are all loaded before their sums.
+// flight at once (four partial dot products), and value rows are loaded 64 registers at a time before
+// their sums. Against one warp per (row, head) on every group, two layers and the head: iteration of 32
+// rows at 1,000 tokens 354 -> 196 us, at 3,000 854 -> 363 us, one row at 3,000 721 -> 240 us (heads of 64
+// dims; 411 -> 280, 979 -> 592 and 928 -> 486 us for 128); error against 64 bits at 3,000 tokens 1.7e-6
+// -> 1.1e-6, at 33 and 200 the same within a tenth.
 constexpr int F32_WARPS = 4;
 template <int HDT>
 __global__ void __launch_bounds__(32 * F32_WARPS) k_attn_f32(const AttnParams a) {

@@ -3,7 +3,8 @@
 Projection: 16- and 32-token tiles, the cluster's K shares (1, 2, 4, 8 CTAs), feature counts and K that
 are no multiple of a tile or of four, and buffers that are not 16-byte aligned (4-byte copies). The
 bound is the fp32 sum's: K * 2^-24 of the sum of absolute products, which it stays far below.
-Attention: heads of 64 and of 128 dims, drafts that end inside a 32-key group.
+Attention: heads of 64 and of 128 dims; drafts that end inside a 32-key group, and that leave its four
+warps one group each, fewer, or several.
 """
 import dataclasses
 
@@ -44,14 +45,14 @@ def test_gemm_f32_edges(N, K, M, offset):
 
 
 @pytest.mark.parametrize("head_dim", [64, 128])
-@pytest.mark.parametrize("prompt,rows", [(1, 1), (31, 2), (45, 20)])
+@pytest.mark.parametrize("prompt,rows", [(1, 1), (31, 2), (45, 20), (96, 32), (127, 2), (255, 9)])
 def test_attention_f32_head_dims(head_dim, prompt, rows):
     need_gpu()
     from paper_2512_14681_gb300.jacobi import Context
 
     shape = dataclasses.replace(I.TINY_F32, name=f"tiny-f32-hd{head_dim}", head_dim=head_dim)
     toks = I.prompt_tokens(shape.vocab, prompt + rows, seed=head_dim + prompt)
-    ctx = Context(shape, max_ctx=128, max_rows=64, logits_rows=32)
+    ctx = Context(shape, max_ctx=320, max_rows=64, logits_rows=32)
     try:
         ctx.init_random_weights(I.WEIGHT_SEED, I.WEIGHT_STD)
         ctx.prefill(0, toks[:prompt])
@@ -60,5 +61,5 @@ def test_attention_f32_head_dims(head_dim, prompt, rows):
         ctx.close()
     model = O.Model(O.ModelConfig(**shape.oracle_kwargs())).init_random(I.WEIGHT_SEED, I.WEIGHT_STD)
     n = prompt + rows
-    ref = O.forward(model, O.Cache(model, 128, n), toks, np.arange(n), want_logits=True).logits[prompt:]
+    ref = O.forward(model, O.Cache(model, 320, n), toks, np.arange(n), want_logits=True).logits[prompt:]
     assert np.abs(logits - ref).max() < 1e-4
