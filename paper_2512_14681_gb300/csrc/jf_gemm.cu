@@ -695,7 +695,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
 // depends on N and K alone. These models' matrices are small (a 256 x 1024 one is two feature tiles), so
 // latency bounds the kernel: it is spread over 8-152 SMs instead of one CTA per tile whose threads each
 // walked a weight row (a jf_op_gemm call of 4096 x 1024, 40 rows: 158 -> 41 us, most of which is now the
-// call itself; the tiny fp32 decoder's generation, with the fp32 attention: 35.6 -> 6.9 ms).
+// call itself; the tiny fp32 decoder's generation, with the fp32 attention: 35.9 -> 6.2 ms).
 // ---------------------------------------------------------------------------------------------
 constexpr int F32_BK = 32;
 constexpr int F32_STAGES = 4;
@@ -739,10 +739,9 @@ __global__ void __launch_bounds__(F32_THREADS) k_gemm_f32(const float* __restric
   const int n0 = n_tile * kTileN, m0 = blockIdx.z * BN;
   const int kb0 = (int)((long long)p.kb_total * split / n_splits), kb1 = (int)((long long)p.kb_total * (split + 1) / n_splits);
   pdl_launch_dependents();
-  pdl_wait();
-  auto load = [&](int kb) {
+  auto load = [&](int kb, int first, int last) {  // rows [first, last) of the stage: weights, then tokens
     const uint32_t base = smem_u32(tiles + ((kb - kb0) % F32_STAGES) * f32_stage_floats(BN));
-    for (int i = tid; i < (kTileN + BN) * (F32_BK / 4); i += F32_THREADS) {
+    for (int i = first * (F32_BK / 4) + tid; i < last * (F32_BK / 4); i += F32_THREADS) {
       const int r = i / (F32_BK / 4), c = (i % (F32_BK / 4)) * 4;
       const bool w = r < kTileN;
       const int g = w ? n0 + r : m0 + r - kTileN;
@@ -751,8 +750,17 @@ __global__ void __launch_bounds__(F32_THREADS) k_gemm_f32(const float* __restric
                 vec);
     }
   };
+  // A forward's weights were complete before it began: their first tiles are fetched before the
+  // dependency wait (the tiny decoder's generation 6.63 -> 6.23 ms). jf_op_gemm's W may be the previous
+  // call's Y, so EPI_STORE waits first.
+  constexpr bool kEarly = EPI != EPI_STORE;
+  if (kEarly) {
+    for (int s = 0; s < F32_STAGES - 1; ++s)
+      if (kb0 + s < kb1) load(kb0 + s, 0, kTileN);
+  }
+  pdl_wait();
   for (int s = 0; s < F32_STAGES - 1; ++s) {
-    if (kb0 + s < kb1) load(kb0 + s);
+    if (kb0 + s < kb1) load(kb0 + s, kEarly ? kTileN : 0, kTileN + BN);
     asm volatile("cp.async.commit_group;" ::: "memory");
   }
   float acc[BN];
@@ -761,7 +769,7 @@ __global__ void __launch_bounds__(F32_THREADS) k_gemm_f32(const float* __restric
   for (int kb = kb0; kb < kb1; ++kb) {
     asm volatile("cp.async.wait_group %0;" ::"n"(F32_STAGES - 2) : "memory");
     __syncthreads();  // this tile has landed; the one before it has been read by everyone
-    if (kb + F32_STAGES - 1 < kb1) load(kb + F32_STAGES - 1);
+    if (kb + F32_STAGES - 1 < kb1) load(kb + F32_STAGES - 1, 0, kTileN + BN);
     asm volatile("cp.async.commit_group;" ::: "memory");
     const float* wt = tiles + ((kb - kb0) % F32_STAGES) * f32_stage_floats(BN) + half * (F32_BK / 2);
     const float* xt = wt + kTileN * F32_PITCH;
