@@ -145,6 +145,12 @@ cudaError_t launch_gemm_bf16(const CUtensorMap& tmA, const CUtensorMap& tmB, con
 cudaError_t launch_gemm_f32(const float* W, const float* X, const GemmParams& p, cudaStream_t st);
 int gemm_bn_for(int M);
 int gemm_box_rows(int bn);
+// Bytes of jf_op_gemm's split-K partial tiles. A 16-token tile is given a 32-token one's room: the size
+// that a caller has allocated, and the shapes that the fixed scratch of jf_op_gemm_noalloc takes, are
+// the same for every count up to 32 rows.
+inline size_t gemm_partial_bytes(int n_tiles, int m_tiles, int k_splits, int bn) {
+  return k_splits > 1 ? (size_t)n_tiles * m_tiles * k_splits * (bn < 32 ? 32 : bn) * kTileN * 4 : 0;
+}
 #ifdef JF_TIMELINE
 // Timeline builds: point each translation unit's record buffer / counter at caller memory.
 cudaError_t tl_set_gemm(void* records, void* counter);

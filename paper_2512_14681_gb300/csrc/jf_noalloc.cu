@@ -58,7 +58,7 @@ extern "C" jf_status jf_op_gemm_noalloc(const void* W, const void* X, float* Y, 
   const int nt = (N + kTileN - 1) / kTileN, mt = (M + bn - 1) / bn, kb = (K + kTileK - 1) / kTileK;
   int sp = k_splits > 0 ? (k_splits < kb ? k_splits : kb) : gemm_default_splits(nt, kb);
   if (sp > 8) sp = 8;
-  const size_t partial_bytes = sp > 1 ? (size_t)nt * mt * sp * bn * kTileN * 4 : 0;
+  const size_t partial_bytes = gemm_partial_bytes(nt, mt, sp, bn);
   int* tickets = reinterpret_cast<int*>(reinterpret_cast<char*>(scratch) + rup256(partial_bytes));
   cudaStream_t st = reinterpret_cast<cudaStream_t>(cuda_stream);
   // the array keeps the previous call's contents: the tickets must start at zero

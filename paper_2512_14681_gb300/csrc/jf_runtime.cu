@@ -1584,7 +1584,7 @@ jf_status jf_op_gemm_workspace_bytes(int N, int K, int M, int k_splits, size_t* 
   if (N < 1 || K < 1 || M < 1 || !out) return JF_EINVAL;
   int bn, nt, mt, kb, sp;
   op_gemm_shape(JF_BF16, N, K, M, k_splits, &bn, &nt, &mt, &kb, &sp);
-  const size_t partial = sp > 1 ? (size_t)nt * mt * sp * bn * kTileN * 4 : 0;
+  const size_t partial = gemm_partial_bytes(nt, mt, sp, bn);
   *out = rup(partial, 256) + rup((size_t)nt * mt * 4, 256);
   return JF_OK;
 }
@@ -1611,7 +1611,7 @@ jf_status jf_op_gemm(int dtype, const void* W, const void* X, float* Y, int N, i
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     p.grid = sms;
   }
-  const size_t partial = sp > 1 ? (size_t)nt * mt * sp * bn * kTileN * 4 : 0;
+  const size_t partial = gemm_partial_bytes(nt, mt, sp, bn);
   p.ws = reinterpret_cast<float*>(workspace);
   p.tile_counter = workspace ? reinterpret_cast<int*>(reinterpret_cast<char*>(workspace) + rup(partial, 256)) : nullptr;
   p.err = err_word;
