@@ -68,7 +68,7 @@ struct CommitInfo {
   int row0, k, P;
 };
 
-// Result copied to pinned host memory after every iteration.
+// Result of an iteration, written to pinned host memory.
 struct IterResult {
   int next_M;
   int n_chains;
@@ -98,6 +98,25 @@ struct StepResult {
   int q0_next;
   int counts[kMaxStepBlocks];
 };
+
+// 4-byte words copied between device memory and pinned host memory by one kernel.
+constexpr int kMaxWordCopies = 6;
+struct WordCopies {
+  int n_copies = 0;
+  const int* src[kMaxWordCopies];
+  int* dst[kMaxWordCopies];
+  int n[kMaxWordCopies];
+  void add(const void* s, void* d, size_t bytes) {
+    src[n_copies] = static_cast<const int*>(s);
+    dst[n_copies] = static_cast<int*>(d);
+    n[n_copies++] = (int)(bytes / 4);
+  }
+};
+cudaError_t launch_copy_words(const WordCopies& w, cudaStream_t st);
+// Rows of a forward of one causal chain: tokens (pinned host or device), positions P .. P+M-1, the chain
+// table, and the commit entry of the whole chain.
+cudaError_t launch_set_chain(const int* tokens, int seq, int P, int M, int* tok, int* pos, Chain* chains, int* n_chains,
+                             CommitInfo* commit, cudaStream_t st);
 
 cudaError_t launch_gen_init(const GenCfg& g, int* state, const int* q0, const int* seq_len, const int* prompt_last,
                             int* tok, int* pos, Chain* chains, int* n_chains_dev, IterResult* res, int* err,

@@ -127,7 +127,7 @@ struct Offsets {
   size_t tok, pos, gpred, top2, chains, n_chains, attn_xchg;
   size_t gemm_ws, gemm_counter, am_v1, am_i1, am_v2;
   size_t logits, err, traj_count;
-  size_t gen_state, gen_out, gen_truth, gen_log, gen_q0, gen_plast, gen_prompt, gen_seqp, res, step_blocks, step_res,
+  size_t gen_state, gen_out, gen_truth, gen_log, gen_q0, gen_plast, gen_prompt, gen_seqp, step_blocks, step_res,
       committed;
   size_t gemm_ws_bytes;
   size_t total;
@@ -260,7 +260,6 @@ Offsets plan_offsets(const Dims& D) {
   o.gen_plast = p.take((size_t)D.S * 4);
   o.gen_prompt = p.take((size_t)D.S * D.max_ctx * 4);
   o.gen_seqp = p.take((size_t)D.S * kSeqParams * 4);
-  o.res = p.take(sizeof(IterResult));
   o.step_blocks = p.take(sizeof(StepBlocks));
   o.step_res = p.take(sizeof(StepResult));
   o.committed = p.take((size_t)D.R * 4);
@@ -329,12 +328,13 @@ struct jf_ctx {
   float* logits;
   int* err;
   int *gen_state, *gen_out, *gen_truth, *gen_log, *gen_q0, *gen_plast, *gen_prompt, *gen_seqp, *traj_count;
-  IterResult* res_dev;
   StepBlocks* sb_dev;
   StepResult* sres_dev;
   int* committed_dev;
   // pinned host
   IterResult* res_host = nullptr;
+  int* words_in = nullptr;   // what a call's first kernel reads: a prompt, or a step's rows and tables
+  int* words_out = nullptr;  // what its last kernel writes: the error word, then results
   // host mirrors
   std::vector<int> h_seq_len;
   std::vector<std::vector<int>> h_pages;
@@ -379,16 +379,27 @@ jf_status check_err_word(jf_ctx* c, int code) {
   return fail(c, JF_EDEVICE, "device bounds check failed (code " + std::to_string(code) + ")");
 }
 
-jf_status read_err(jf_ctx* c) {
-  int e = 0;
-  CK(cudaMemcpyAsync(&e, c->err, 4, cudaMemcpyDeviceToHost, c->st));
-  CK(cudaStreamSynchronize(c->st));
+void free_pinned(jf_ctx* c) {
+  if (c->res_host) cudaFreeHost(c->res_host);
+  if (c->words_in) cudaFreeHost(c->words_in);
+  if (c->words_out) cudaFreeHost(c->words_out);
+}
+
+// The error word that the stream's work left, read with it (the stream is idle); a set one is cleared.
+jf_status take_err(jf_ctx* c, int e) {
   if (e) {
     int z = 0;
     cudaMemcpyAsync(c->err, &z, 4, cudaMemcpyHostToDevice, c->st);
     cudaStreamSynchronize(c->st);
   }
   return check_err_word(c, e);
+}
+
+jf_status read_err(jf_ctx* c) {
+  int e = 0;
+  CK(cudaMemcpyAsync(&e, c->err, 4, cudaMemcpyDeviceToHost, c->st));
+  CK(cudaStreamSynchronize(c->st));
+  return take_err(c, e);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -598,18 +609,10 @@ cudaError_t enqueue_forward(jf_ctx* c, int M, LmMode lm) {
   return gemm(c, c->tm_lm, c->w_lm, c->h, D.V, D.d, lm_rows, el, PC_LMHEAD);
 }
 
-// Upload the rows of one causal chain of sequence `seq` (positions P .. P+M-1).
-jf_status upload_chain(jf_ctx* c, int seq, int P, int M, const int32_t* tokens_host, const int32_t* tokens_dev) {
-  std::vector<int> pos(M);
-  for (int i = 0; i < M; ++i) pos[i] = P + i;
-  Chain ch{seq, 0, M, P};
-  int one = 1;
-  if (tokens_dev) CK(cudaMemcpyAsync(c->tok, tokens_dev, (size_t)M * 4, cudaMemcpyDeviceToDevice, c->st));
-  else CK(cudaMemcpyAsync(c->tok, tokens_host, (size_t)M * 4, cudaMemcpyHostToDevice, c->st));
-  CK(cudaMemcpyAsync(c->pos, pos.data(), (size_t)M * 4, cudaMemcpyHostToDevice, c->st));
-  CK(cudaMemcpyAsync(c->chains, &ch, sizeof(Chain), cudaMemcpyHostToDevice, c->st));
-  CK(cudaMemcpyAsync(c->n_chains, &one, 4, cudaMemcpyHostToDevice, c->st));
-  CK(cudaStreamSynchronize(c->st));
+// Set the rows of one causal chain of sequence `seq` (positions P .. P+M-1). Host tokens lie in words_in.
+jf_status set_chain(jf_ctx* c, int seq, int P, int M, const int32_t* tokens) {
+  CK(launch_set_chain(tokens, seq, P, M, c->tok, c->pos, c->chains, c->n_chains, c->commit + seq, c->st));
+  c->launches += 1;
   c->chains_bound = 1;
   return JF_OK;
 }
@@ -627,28 +630,31 @@ jf_status prefill_impl(jf_ctx* c, int seq, const int32_t* host_prompt, const int
   const int P0 = c->h_seq_len[seq];
   jf_status s;
   if ((s = ensure_pages(c, seq, P0 + len)) != JF_OK) return s;
+  const int32_t* prompt = dev_prompt;
+  if (host_prompt) {
+    std::memcpy(c->words_in, host_prompt, (size_t)len * 4);
+    prompt = c->words_in;
+  }
   int P = P0;
   for (int start = 0; start < len; start += D.R) {
     const int m = std::min(D.R, len - start);
-    s = upload_chain(c, seq, P, m, host_prompt ? host_prompt + start : nullptr, dev_prompt ? dev_prompt + start : nullptr);
-    if (s != JF_OK) return s;
+    if ((s = set_chain(c, seq, P, m, prompt + start)) != JF_OK) return s;
     const bool last_chunk = start + m >= len;
     CK(enqueue_forward(c, m, last_chunk ? LM_LAST : LM_NONE));
-    CommitInfo ci{0, m, P};
-    CK(cudaMemcpyAsync(c->commit + seq, &ci, sizeof(ci), cudaMemcpyHostToDevice, c->st));
     CK(launch_commit(c->commit + seq, 1, m, D.L, c->k_inf, c->v_inf, c->k_pages, c->v_pages,
                      c->page_table + (size_t)seq * D.pps, D.pps, D.n_pages, D.R, D.Hkv, D.hd, D.es, c->seq_len + seq,
                      c->err, c->st));
     c->launches += 1;
     P += m;
-    if (start + m >= len) {
-      int32_t q0 = -1;
-      CK(cudaMemcpyAsync(&q0, c->gpred, 4, cudaMemcpyDeviceToHost, c->st));
-      CK(cudaStreamSynchronize(c->st));
-      if (next) *next = q0;
-    }
   }
-  if ((s = read_err(c)) != JF_OK) return s;
+  WordCopies out;
+  out.add(c->err, c->words_out, 4);
+  out.add(c->gpred, c->words_out + 1, 4);
+  CK(launch_copy_words(out, c->st));
+  c->launches += 1;
+  CK(cudaStreamSynchronize(c->st));
+  if (next) *next = c->words_out[1];
+  if ((s = take_err(c, c->words_out[0])) != JF_OK) return s;
   c->h_seq_len[seq] = P;
   return JF_OK;
 }
@@ -661,7 +667,7 @@ cudaError_t enqueue_iteration(jf_ctx* c, const GenCfg& g, int M, int n_seqs) {
   cudaError_t e = enqueue_forward(c, M, LM_ARGMAX);
   if (e != cudaSuccess) return e;
   prof_begin(c, PC_OTHER);
-  e = launch_gen_accept(g, c->gen_state, c->gpred, M, c->tok, c->pos, c->chains, c->n_chains, c->commit, c->res_dev,
+  e = launch_gen_accept(g, c->gen_state, c->gpred, M, c->tok, c->pos, c->chains, c->n_chains, c->commit, c->res_host,
                         c->err, c->st);
   prof_end(c);
   if (e != cudaSuccess) return e;
@@ -671,7 +677,7 @@ cudaError_t enqueue_iteration(jf_ctx* c, const GenCfg& g, int M, int n_seqs) {
   prof_end(c);
   if (e != cudaSuccess) return e;
   c->launches += 2;
-  return cudaMemcpyAsync(c->res_host, c->res_dev, sizeof(IterResult), cudaMemcpyDeviceToHost, c->st);
+  return cudaSuccess;
 }
 
 bool same_cfg(const GenCfg& a, const GenCfg& b) { return std::memcmp(&a, &b, sizeof(GenCfg)) == 0; }
@@ -906,9 +912,8 @@ jf_status generate_impl(jf_ctx* c, int n_seqs, const int32_t* const* h_prompts, 
     CK(cudaMemsetAsync(c->traj_count, 0, 4, c->st));
   }
   CK(launch_gen_init(g, c->gen_state, c->gen_q0, c->seq_len, c->gen_plast, c->tok, c->pos, c->chains, c->n_chains,
-                     c->res_dev, c->err, c->st));
+                     c->res_host, c->err, c->st));
   c->launches += 1;
-  CK(cudaMemcpyAsync(c->res_host, c->res_dev, sizeof(IterResult), cudaMemcpyDeviceToHost, c->st));
   CK(cudaStreamSynchronize(c->st));
   jf_status s = check_err_word(c, c->res_host->err);
   if (s != JF_OK) return s;
@@ -1008,7 +1013,7 @@ jf_status jf_create(const jf_model_config* model, const jf_runtime_config* rt, j
   }
   // a failure from here on releases what the context already holds
   auto abandon = [c](jf_status s) {
-    if (c->res_host) cudaFreeHost(c->res_host);
+    free_pinned(c);
     if (c->own_stream) cudaStreamDestroy(c->st);
     delete c;
     return s;
@@ -1086,14 +1091,17 @@ jf_status jf_create(const jf_model_config* model, const jf_runtime_config* rt, j
   c->traj_count = at<int>(c, O.traj_count);
   c->gen_prompt = at<int>(c, O.gen_prompt);
   c->gen_seqp = at<int>(c, O.gen_seqp);
-  c->res_dev = at<IterResult>(c, O.res);
   c->sb_dev = at<StepBlocks>(c, O.step_blocks);
   c->sres_dev = at<StepResult>(c, O.step_res);
   c->committed_dev = at<int>(c, O.committed);
-  if (cudaMallocHost(&c->res_host, sizeof(IterResult)) != cudaSuccess) {
-    c->res_host = nullptr;
+  // pinned host memory: an iteration's result, a call's inputs (a prompt or one step) and outputs
+  const size_t in_words = std::max<size_t>((size_t)c->D.pps * kPage, 2 * (size_t)c->D.R + 4 * (size_t)c->D.max_chains + 1 +
+                                                                         sizeof(StepBlocks) / 4);
+  const size_t out_words = 1 + sizeof(StepResult) / 4 + 4 * (size_t)c->D.R;
+  if (cudaMallocHost(&c->res_host, sizeof(IterResult)) != cudaSuccess ||
+      cudaMallocHost(&c->words_in, in_words * 4) != cudaSuccess ||
+      cudaMallocHost(&c->words_out, out_words * 4) != cudaSuccess)
     return abandon(JF_ENOMEM);
-  }
   init_pages(c);
   // zero the small control buffers; fill the page table with -1
   cudaError_t e = cudaSuccess;
@@ -1123,7 +1131,7 @@ void jf_destroy(jf_ctx* c) {
   if (!c) return;
   if (c->st) cudaStreamSynchronize(c->st);
   drop_graphs(c);
-  if (c->res_host) cudaFreeHost(c->res_host);
+  free_pinned(c);
   if (c->own_stream) cudaStreamDestroy(c->st);
   delete c;
 }
@@ -1428,12 +1436,20 @@ jf_status jf_jacobi_step(jf_ctx* c, int seq, int n_blocks, const jf_block* block
   if (s != JF_OK) return s;
   if ((s = ensure_pages(c, seq, max_pos)) != JF_OK) return s;
   const int nch = (int)chains.size();
-  CK(cudaMemcpyAsync(c->tok, draft, (size_t)total * 4, cudaMemcpyHostToDevice, c->st));
-  CK(cudaMemcpyAsync(c->pos, pos.data(), (size_t)total * 4, cudaMemcpyHostToDevice, c->st));
-  CK(cudaMemcpyAsync(c->chains, chains.data(), (size_t)nch * sizeof(Chain), cudaMemcpyHostToDevice, c->st));
-  CK(cudaMemcpyAsync(c->n_chains, &nch, 4, cudaMemcpyHostToDevice, c->st));
-  CK(cudaMemcpyAsync(c->sb_dev, &sb, sizeof(sb), cudaMemcpyHostToDevice, c->st));
-  CK(cudaStreamSynchronize(c->st));
+  WordCopies in, res;
+  int* w = c->words_in;
+  auto stage = [&](const void* src, void* dst, size_t bytes) {
+    std::memcpy(w, src, bytes);
+    in.add(w, dst, bytes);
+    w += bytes / 4;
+  };
+  stage(draft, c->tok, (size_t)total * 4);
+  stage(pos.data(), c->pos, (size_t)total * 4);
+  stage(chains.data(), c->chains, (size_t)nch * sizeof(Chain));
+  stage(&nch, c->n_chains, 4);
+  stage(&sb, c->sb_dev, sizeof(sb));
+  CK(launch_copy_words(in, c->st));
+  c->launches += 1;
   c->chains_bound = nch;
   CK(enqueue_forward(c, total, LM_ARGMAX));
   CK(launch_step_accept(c->sb_dev, c->tok, c->gpred, c->committed_dev, c->commit, c->sres_dev, c->err, c->st));
@@ -1441,13 +1457,24 @@ jf_status jf_jacobi_step(jf_ctx* c, int seq, int n_blocks, const jf_block* block
                    c->page_table + (size_t)seq * D.pps, D.pps, D.n_pages, D.R, D.Hkv, D.hd, D.es, c->seq_len + seq,
                    c->err, c->st));
   StepResult r;
-  CK(cudaMemcpyAsync(&r, c->sres_dev, sizeof(r), cudaMemcpyDeviceToHost, c->st));
-  if (predictions) CK(cudaMemcpyAsync(predictions, c->gpred, (size_t)total * 4, cudaMemcpyDeviceToHost, c->st));
-  if (top2) CK(cudaMemcpyAsync(top2, c->top2, (size_t)total * 8, cudaMemcpyDeviceToHost, c->st));
+  int* const r_host = c->words_out + 1;
+  int* const pred_host = r_host + sizeof(StepResult) / 4;
+  int* const top2_host = pred_host + D.R;
+  int* const comm_host = top2_host + 2 * (size_t)D.R;
+  res.add(c->err, c->words_out, 4);
+  res.add(c->sres_dev, r_host, sizeof(StepResult));
+  res.add(c->committed_dev, comm_host, (size_t)max_len * 4);
+  if (predictions) res.add(c->gpred, pred_host, (size_t)total * 4);
+  if (top2) res.add(c->top2, top2_host, (size_t)total * 8);
+  CK(launch_copy_words(res, c->st));
+  c->launches += 1;
   CK(cudaStreamSynchronize(c->st));
-  if ((s = read_err(c)) != JF_OK) return s;
+  std::memcpy(&r, r_host, sizeof(r));
+  if (predictions) std::memcpy(predictions, pred_host, (size_t)total * 4);
+  if (top2) std::memcpy(top2, top2_host, (size_t)total * 8);
+  if ((s = take_err(c, c->words_out[0])) != JF_OK) return s;
   if (r.k < 1 || r.k > max_len) return fail(c, JF_EDEVICE, "invalid accepted count");
-  CK(cudaMemcpy(committed_tokens, c->committed_dev, (size_t)r.k * 4, cudaMemcpyDeviceToHost));
+  std::memcpy(committed_tokens, comm_host, (size_t)r.k * 4);
   for (int b = 0; b < n_blocks; ++b) accepted_counts[b] = r.counts[b];
   *n_committed = r.k;
   c->h_seq_len[seq] = P + r.k;
@@ -1466,9 +1493,9 @@ jf_status jf_forward_logits(jf_ctx* c, int seq, int n_rows, const int32_t* token
   if (P + n_rows > D.max_ctx) return fail(c, JF_ECAPACITY, "positions beyond max_ctx");
   jf_status s = check_tokens(c, tokens, n_rows);
   if (s != JF_OK) return s;
-  if ((s = upload_chain(c, seq, P, n_rows, tokens, nullptr)) != JF_OK) return s;
+  std::memcpy(c->words_in, tokens, (size_t)n_rows * 4);
+  if ((s = set_chain(c, seq, P, n_rows, c->words_in)) != JF_OK) return s;
   CK(enqueue_forward(c, n_rows, LM_ARGMAX));
-  if (argmax) CK(cudaMemcpyAsync(argmax, c->gpred, (size_t)n_rows * 4, cudaMemcpyDeviceToHost, c->st));
   if (logits) {
     // the LM head again, storing the logits instead of reducing them
     GemmEpi el = {};
@@ -1476,11 +1503,19 @@ jf_status jf_forward_logits(jf_ctx* c, int seq, int n_rows, const int32_t* token
     el.y = c->logits;
     el.ldy = D.V;
     CK(gemm(c, c->tm_lm, c->w_lm, c->h, D.V, D.d, n_rows, el, -1));
+  }
+  WordCopies out;
+  out.add(c->err, c->words_out, 4);
+  out.add(c->gpred, c->words_out + 1, (size_t)n_rows * 4);
+  CK(launch_copy_words(out, c->st));
+  c->launches += 1;
+  if (logits) {
     CK(cudaMemcpyAsync(logits, c->logits, (size_t)n_rows * D.V * 4, cudaMemcpyDeviceToHost, c->st));
   }
   if (hidden) CK(cudaMemcpyAsync(hidden, c->x, (size_t)n_rows * D.d * 4, cudaMemcpyDeviceToHost, c->st));
   CK(cudaStreamSynchronize(c->st));
-  return read_err(c);
+  if (argmax) std::memcpy(argmax, c->words_out + 1, (size_t)n_rows * 4);
+  return take_err(c, c->words_out[0]);
 }
 
 jf_status jf_generate(jf_ctx* c, int n_seqs, const int32_t* const* prompts, const int32_t* prompt_lens,
