@@ -678,7 +678,7 @@ __global__ void __launch_bounds__(256) k_set_chain(const int* __restrict__ token
                                                    Chain* chains, int* n_chains, CommitInfo* commit) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < M) {
-    tok[i] = tokens[i];
+    if (tokens) tok[i] = tokens[i];
     pos[i] = P + i;
   }
   if (i == 0) {

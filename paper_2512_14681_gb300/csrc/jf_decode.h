@@ -113,8 +113,8 @@ struct WordCopies {
   }
 };
 cudaError_t launch_copy_words(const WordCopies& w, cudaStream_t st);
-// Rows of a forward of one causal chain: tokens (pinned host or device), positions P .. P+M-1, the chain
-// table, and the commit entry of the whole chain.
+// Rows of a forward of one causal chain: tokens (in pinned host memory; null when they are in `tok`
+// already), positions P .. P+M-1, the chain table, and the commit entry of the whole chain.
 cudaError_t launch_set_chain(const int* tokens, int seq, int P, int M, int* tok, int* pos, Chain* chains, int* n_chains,
                              CommitInfo* commit, cudaStream_t st);
 

@@ -609,8 +609,10 @@ cudaError_t enqueue_forward(jf_ctx* c, int M, LmMode lm) {
   return gemm(c, c->tm_lm, c->w_lm, c->h, D.V, D.d, lm_rows, el, PC_LMHEAD);
 }
 
-// Set the rows of one causal chain of sequence `seq` (positions P .. P+M-1). Host tokens lie in words_in.
-jf_status set_chain(jf_ctx* c, int seq, int P, int M, const int32_t* tokens) {
+// Set the rows of one causal chain of sequence `seq` (positions P .. P+M-1): host tokens lie in words_in,
+// a caller's device tokens are copied (they may have any alignment).
+jf_status set_chain(jf_ctx* c, int seq, int P, int M, const int32_t* tokens, const int32_t* tokens_dev) {
+  if (tokens_dev) CK(cudaMemcpyAsync(c->tok, tokens_dev, (size_t)M * 4, cudaMemcpyDeviceToDevice, c->st));
   CK(launch_set_chain(tokens, seq, P, M, c->tok, c->pos, c->chains, c->n_chains, c->commit + seq, c->st));
   c->launches += 1;
   c->chains_bound = 1;
@@ -630,15 +632,12 @@ jf_status prefill_impl(jf_ctx* c, int seq, const int32_t* host_prompt, const int
   const int P0 = c->h_seq_len[seq];
   jf_status s;
   if ((s = ensure_pages(c, seq, P0 + len)) != JF_OK) return s;
-  const int32_t* prompt = dev_prompt;
-  if (host_prompt) {
-    std::memcpy(c->words_in, host_prompt, (size_t)len * 4);
-    prompt = c->words_in;
-  }
+  if (host_prompt) std::memcpy(c->words_in, host_prompt, (size_t)len * 4);
   int P = P0;
   for (int start = 0; start < len; start += D.R) {
     const int m = std::min(D.R, len - start);
-    if ((s = set_chain(c, seq, P, m, prompt + start)) != JF_OK) return s;
+    s = set_chain(c, seq, P, m, host_prompt ? c->words_in + start : nullptr, dev_prompt ? dev_prompt + start : nullptr);
+    if (s != JF_OK) return s;
     const bool last_chunk = start + m >= len;
     CK(enqueue_forward(c, m, last_chunk ? LM_LAST : LM_NONE));
     CK(launch_commit(c->commit + seq, 1, m, D.L, c->k_inf, c->v_inf, c->k_pages, c->v_pages,
@@ -1494,7 +1493,7 @@ jf_status jf_forward_logits(jf_ctx* c, int seq, int n_rows, const int32_t* token
   jf_status s = check_tokens(c, tokens, n_rows);
   if (s != JF_OK) return s;
   std::memcpy(c->words_in, tokens, (size_t)n_rows * 4);
-  if ((s = set_chain(c, seq, P, n_rows, c->words_in)) != JF_OK) return s;
+  if ((s = set_chain(c, seq, P, n_rows, c->words_in, nullptr)) != JF_OK) return s;
   CK(enqueue_forward(c, n_rows, LM_ARGMAX));
   if (logits) {
     // the LM head again, storing the logits instead of reducing them
