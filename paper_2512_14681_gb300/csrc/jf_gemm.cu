@@ -5,7 +5,7 @@
 // the (few) in-flight tokens its N side. A persistent, warp-specialised kernel: one CTA per SM
 // walks its share of (tile, split) work units; a producer warp streams weight and activation
 // tiles by TMA (128-byte swizzle) through a 4-12 stage mbarrier ring that never drains between
-// units; an MMA warp accumulates into one of two TMEM accumulators; four epilogue warps drain
+// units; an MMA warp accumulates into one of two TMEM accumulators; eight epilogue warps drain
 // the other accumulator (fused epilogue, split-K reduction) while the next unit streams in.
 // fp32 path (small fp32 models): a SIMT mainloop over 128-feature tiles with the same epilogues.
 //
@@ -392,9 +392,9 @@ JF_DEV Unit unit_of(const GemmParams& p, int u) {
 // eight warps halve it), warp 8 = TMA producer, warp 9 = MMA issuer (and the TMEM allocation).
 // (8 layers and head of the 7B shape: 64 rows 990 -> 978 us, 160 rows 1198 -> 1167; 32 rows as before).
 //
-// PAIR (256-token tiles, i.e. more than 160 rows): two CTAs on neighbouring SMs take a tile of 256
-// weight rows together (cta_group::2). Each loads its own 128 weight rows and half of the tokens (32 KB
-// a 64-k stage instead of 48), rank 0 issues the MMAs of both, and each drains its own 128 rows. With
+// PAIR (more than 160 rows): two CTAs on neighbouring SMs take a tile of 256 weight rows together
+// (cta_group::2). Each loads its own 128 weight rows and half of the tokens (at 256 tokens 32 KB a 64-k
+// stage instead of 48), rank 0 issues the MMAs of both, and each drains its own 128 rows. With
 // one CTA per tile the operands, not the tensor cores, bounded it: 48 KB a 512-cycle stage is more than
 // an SM draws from L2, and only four such stages fit. gate/up (37888 x 3584) at 512 rows: 110.6 ->
 // 104.9 us a call (1.33 PFLOP/s); prefill of 4,000 tokens through one 7B layer 2.39 -> 2.29 ms.
@@ -907,6 +907,9 @@ static cudaError_t gemm_prepare_current() {
   if ((e = prep_tc<64>()) != cudaSuccess) return e;
   if ((e = prep_tc<128>()) != cudaSuccess) return e;
   if ((e = prep_tc<160>()) != cudaSuccess) return e;
+  if ((e = prep_tc<160, true>()) != cudaSuccess) return e;
+  if ((e = prep_tc<192, true>()) != cudaSuccess) return e;
+  if ((e = prep_tc<224, true>()) != cudaSuccess) return e;
   return prep_tc<256, true>();
 }
 
@@ -921,38 +924,28 @@ cudaError_t gemm_prepare() {
   return r < 0 ? cudaErrorInvalidDevice : static_cast<cudaError_t>(r);
 }
 
-// Token-tile width: the narrowest tile that holds every row (16 columns leave room for twelve stages
-// instead of ten and halve the activation copies: one row of the 7B shape, 8 layers and head, 879 -> 867 us
-// against a 32-wide tile, 16 rows 908 -> 905). Above 256 rows the rows take as few tiles as 256-wide
-// ones would (every extra tile is one more pass over the weights), and among the widths that give
-// that count the narrowest (the tensor cores' work grows with the padded rows): 320 rows = 2 x 160,
-// 384 = 2 x 256 (3 x 128 measured slower), 512 = 2 x 256.
+// Token-tile width. Up to 256 rows one tile, the narrowest that holds them; above, as few tiles as 256-wide
+// ones would be (every further tile is another pass over the weights) and among the widths that give that
+// count the narrowest (the tensor cores' work grows with the padded rows). 8 layers and head of the 7B
+// shape, us: 16-wide against 32-wide tiles at one row 867 / 879 (twelve stages instead of ten, half the
+// activation copies); 192 against 256 at 192 rows 1248 / 1275, at 384 (two tiles) 1750 / 1899; 224 against
+// 256 at 224 rows 1293 / 1308, at 448 1900 / 1990. Three 128-wide tiles at 384 rows were slower than two of
+// 256.
 int gemm_bn_for(int M) {
   if (M <= 16) return 16;
   if (M <= 32) return 32;
   if (M <= 64) return 64;
   if (M <= 128) return 128;
-  if (M <= 160) return 160;
-  if (M <= 256) return 256;
   const int tiles = (M + 255) / 256;
-  for (int bn : {128, 160})
+  for (int bn : {128, 160, 192, 224})
     if ((M + bn - 1) / bn == tiles) return bn;
   return 256;
 }
 
-// Token rows of one TMA box of the activations: a pair's CTAs load half of a 256-token tile each.
-int gemm_box_rows(int bn) { return bn == 256 ? 128 : bn; }
-
-size_t gemm_smem_bytes(int bn) {
-  switch (bn) {
-    case 16: return TcCfg<16, false>::SMEM;
-    case 32: return TcCfg<32, false>::SMEM;
-    case 64: return TcCfg<64, false>::SMEM;
-    case 128: return TcCfg<128, false>::SMEM;
-    case 160: return TcCfg<160, false>::SMEM;
-    default: return TcCfg<256, true>::SMEM;
-  }
-}
+// Token rows of one TMA box of the activations: above 160 rows CTA pairs run, whose CTAs load half of a
+// tile's tokens each (320 rows as two 160-wide tiles: 1568 us by pairs, 1660 by single CTAs; pairs at 32,
+// 64, 128 and 160 rows: 0-1% slower, 3% on the 1.5B shape, whose short projections pay for the cluster).
+int gemm_box_rows(int bn, int M) { return M > 160 ? bn / 2 : bn; }
 
 cudaError_t launch_gemm_bf16(const CUtensorMap& tmA, const CUtensorMap& tmB, const GemmParams& p, int bn,
                              cudaStream_t st) {
@@ -961,7 +954,9 @@ cudaError_t launch_gemm_bf16(const CUtensorMap& tmA, const CUtensorMap& tmB, con
     case 32: return launch_tc<32>(tmA, tmB, p, st);
     case 64: return launch_tc<64>(tmA, tmB, p, st);
     case 128: return launch_tc<128>(tmA, tmB, p, st);
-    case 160: return launch_tc<160>(tmA, tmB, p, st);
+    case 160: return p.M > 160 ? launch_tc<160, true>(tmA, tmB, p, st) : launch_tc<160>(tmA, tmB, p, st);
+    case 192: return launch_tc<192, true>(tmA, tmB, p, st);
+    case 224: return launch_tc<224, true>(tmA, tmB, p, st);
     case 256: return launch_tc<256, true>(tmA, tmB, p, st);
     default: return cudaErrorInvalidValue;
   }

@@ -144,12 +144,13 @@ cudaError_t launch_gemm_bf16(const CUtensorMap& tmA, const CUtensorMap& tmB, con
                              cudaStream_t st);
 cudaError_t launch_gemm_f32(const float* W, const float* X, const GemmParams& p, cudaStream_t st);
 int gemm_bn_for(int M);
-int gemm_box_rows(int bn);
-// Bytes of jf_op_gemm's split-K partial tiles. A 16-token tile is given a 32-token one's room: the size
-// that a caller has allocated, and the shapes that the fixed scratch of jf_op_gemm_noalloc takes, are
-// the same for every count up to 32 rows.
+int gemm_box_rows(int bn, int M);
+// Bytes of jf_op_gemm's split-K partial tiles. 16-token tiles are given the room of 32-token ones, 192 and
+// 224 that of 256: the size that a caller has allocated, and the shapes that the fixed scratch of
+// jf_op_gemm_noalloc takes, do not depend on how finely the tile follows the row count.
 inline size_t gemm_partial_bytes(int n_tiles, int m_tiles, int k_splits, int bn) {
-  return k_splits > 1 ? (size_t)n_tiles * m_tiles * k_splits * (bn < 32 ? 32 : bn) * kTileN * 4 : 0;
+  const int room = bn < 32 ? 32 : (bn > 160 ? 256 : bn);
+  return k_splits > 1 ? (size_t)n_tiles * m_tiles * k_splits * room * kTileN * 4 : 0;
 }
 #ifdef JF_TIMELINE
 // Timeline builds: point each translation unit's record buffer / counter at caller memory.
@@ -158,7 +159,6 @@ cudaError_t tl_set_attn(void* records, void* counter);
 cudaError_t tl_set_elem(void* records, void* counter);
 cudaError_t tl_set_decode(void* records, void* counter);
 #endif
-size_t gemm_smem_bytes(int bn);
 int gemm_default_splits(int n_tiles, int kb_total);
 bool encode_tmap_bf16(CUtensorMap* tm, const void* ptr, long long K, long long rows, int box_rows);
 

@@ -87,6 +87,6 @@ extern "C" jf_status jf_op_gemm_noalloc(const void* W, const void* X, float* Y, 
   p.epi.y = Y;
   p.epi.ldy = N;
   CUtensorMap tA, tB;
-  if (!encode_tmap_bf16(&tA, W, K, N, kTileN) || !encode_tmap_bf16(&tB, X, K, M, gemm_box_rows(bn))) return JF_ECUDA;
+  if (!encode_tmap_bf16(&tA, W, K, N, kTileN) || !encode_tmap_bf16(&tB, X, K, M, gemm_box_rows(bn, M))) return JF_ECUDA;
   return launch_gemm_bf16(tA, tB, p, bn, st) == cudaSuccess ? JF_OK : JF_ECUDA;
 }

@@ -501,7 +501,7 @@ cudaError_t gemm(jf_ctx* c, const CUtensorMap& tmA, const void* W, const void* X
     p.m_tiles = cdiv(M, bn);
     p.k_splits = splits_for(p.n_tiles, p.kb_total);
     CUtensorMap tmB;
-    if (!make_tmap(&tmB, X, K, M, gemm_box_rows(bn))) return cudaErrorInvalidValue;
+    if (!make_tmap(&tmB, X, K, M, gemm_box_rows(bn, M))) return cudaErrorInvalidValue;
     e = launch_gemm_bf16(tmA, tmB, p, bn, c->st);
   } else {
     p.k_splits = 1;
@@ -1659,7 +1659,7 @@ jf_status jf_op_gemm(int dtype, const void* W, const void* X, float* Y, int N, i
   if (dtype == JF_BF16) {
     if (gemm_prepare() != cudaSuccess) return JF_ECUDA;  // once per device
     CUtensorMap tA, tB;
-    if (!make_tmap(&tA, W, K, N, kTileN) || !make_tmap(&tB, X, K, M, gemm_box_rows(bn))) return JF_ECUDA;
+    if (!make_tmap(&tA, W, K, N, kTileN) || !make_tmap(&tB, X, K, M, gemm_box_rows(bn, M))) return JF_ECUDA;
     e = launch_gemm_bf16(tA, tB, p, bn, st);
   } else {
     if (gemm_prepare() != cudaSuccess) return JF_ECUDA;

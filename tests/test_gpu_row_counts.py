@@ -1,7 +1,7 @@
 """The bf16 projections, the LM head's argmax and the norms at the row counts where their forms change.
 
-Projection: 16-token tiles up to 16 rows, CTA pairs on 256-token tiles above 160 rows (an odd number of
-128-feature tiles leaves a pair's second CTA without one), reductions that end inside a 128-k stage pair.
+Projection: 16-token tiles up to 16 rows, CTA pairs on tiles of 160 to 256 tokens above 160 rows (an
+odd number of 128-feature tiles leaves a pair's second CTA without one), reductions that end inside a 128-k stage pair.
 Inputs are bf16 values and the reference multiplies them in fp64, so the difference is the fp32 sum's:
 K * 2^-23 of the sum of absolute products (one unit per addition, whichever way it rounds).
 Argmax: in shared memory up to 512 rows, in the CTAs' global slots above; against the stored logits of the
@@ -21,7 +21,7 @@ from tests.parity import need_gpu
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("M", [1, 15, 16, 17, 161, 255, 256, 257, 321])
+@pytest.mark.parametrize("M", [1, 15, 16, 17, 161, 192, 193, 224, 225, 256, 257, 320, 321, 384, 385, 449])
 @pytest.mark.parametrize("N,K,splits", [(1, 8, 0), (129, 64, 0), (384, 192, 0), (128, 72, 0), (640, 1096, 3), (257, 320, 5)])
 def test_gemm_tile_edges(N, K, splits, M):
     torch = need_gpu()
