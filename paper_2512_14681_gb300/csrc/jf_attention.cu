@@ -16,7 +16,8 @@
 // folded in lane order. The tree depends only on absolute key positions, never on how many rows share
 // the forward or how many chunks a unit has, so a row's result is the same in every batch. The lanes
 // of a unit are spread over a cluster of 8, 4 or 2 CTAs, or one CTA takes them all (jf_attn_form.h).
-// fp32 path: one warp per (row, head), keys in absolute order, online softmax in fp32.
+// fp32 path: four warps per (row, head) on absolute 32-key groups, online softmax in fp32, folded in
+// warp order.
 #include "jf_device.cuh"
 #include "jf_internal.h"
 
@@ -65,7 +66,7 @@ JF_DEV float fold_value(float wa, float a, float wb, float b) { return __fmaf_rn
 
 // Unit ui of the forward (chains in order, then KV heads, then query tiles), looked up
 // by warp 0 into s_unit; s_unit.pad stays 0 past the last unit. Every CTA of cluster ui gets the
-// same unit. The chain table was written by host copies or an earlier graph launch, complete
+// same unit. The chain table was written by a kernel or graph launch that was complete
 // before this forward began, so this runs before the dependency wait.
 JF_DEV void resolve_unit(const AttnParams& a, int ui, int j, int n_units, int G, int warp, int lane, AttnUnit& s_unit) {
   if (threadIdx.x == 0) s_unit.pad = 0;
