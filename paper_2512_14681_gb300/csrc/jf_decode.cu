@@ -664,6 +664,19 @@ __global__ void k_commit(const CommitInfo* commit, const uint8_t* k_inf, const u
   pdl_launch_dependents();
 }
 
+cudaLaunchConfig_t pdl_cfg(dim3 grid, dim3 block, size_t smem, cudaStream_t st, cudaLaunchAttribute* at) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cfg;
+}
+
 // Host/device hand-over of a call, a few KB: latency bounds it, so every array goes in one launch (a
 // forward took four copies from pageable memory and a synchronisation before its first kernel, and two
 // copies, each waited for, after its last). One layer of the 7B shape, 32 rows over 1,024 tokens: 181 ->
@@ -686,19 +699,6 @@ __global__ void __launch_bounds__(256) k_set_chain(const int* __restrict__ token
     *n_chains = 1;
     *commit = CommitInfo{0, M, P};
   }
-}
-
-cudaLaunchConfig_t pdl_cfg(dim3 grid, dim3 block, size_t smem, cudaStream_t st, cudaLaunchAttribute* at) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = grid;
-  cfg.blockDim = block;
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  return cfg;
 }
 
 }  // namespace
