@@ -14,7 +14,7 @@
  *     frees caller memory and keeps no pointer to a host buffer after the call returns.
  *   - Device memory: the caller allocates ONE arena of jf_arena_bytes() bytes (e.g. through
  *     PyTorch) and lends it to the context until jf_destroy(). The library allocates no device
- *     memory of its own; it allocates small pinned host buffers for per-iteration results.
+ *     memory of its own; it allocates small pinned host buffers for rows in and results out.
  *   - Work is ordered on the caller's CUDA stream (jf_runtime_config.cuda_stream; NULL lets the
  *     library create a non-blocking stream). Calls that return host outputs synchronise it.
  *   - Every call returns a jf_status. Arguments are validated on the host before any launch; a
