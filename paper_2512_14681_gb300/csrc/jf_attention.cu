@@ -67,7 +67,8 @@ JF_DEV float fold_value(float wa, float a, float wb, float b) { return __fmaf_rn
 // Unit ui of the forward (chains in order, then KV heads, then query tiles), looked up
 // by warp 0 into s_unit; s_unit.pad stays 0 past the last unit. Every CTA of cluster ui gets the
 // same unit. The chain table was written by a kernel or graph launch that was complete
-// before this forward began, so this runs before the dependency wait.
+// before this forward's first kernel (k_embed, no programmatic launch) began, so this runs before the
+// dependency wait.
 JF_DEV void resolve_unit(const AttnParams& a, int ui, int j, int n_units, int G, int warp, int lane, AttnUnit& s_unit) {
   if (threadIdx.x == 0) s_unit.pad = 0;
   __syncthreads();

@@ -681,7 +681,8 @@ cudaLaunchConfig_t pdl_cfg(dim3 grid, dim3 block, size_t smem, cudaStream_t st, 
 // forward took four copies from pageable memory and a synchronisation before its first kernel, and two
 // copies, each waited for, after its last). One layer of the 7B shape, 32 rows over 1,024 tokens: 181 ->
 // 150 us a call; of the 1.5B shape, 19 rows over 777: 118 -> 88; a 4,000-token prefill through one 7B layer
-// 2,213 -> 2,054. No programmatic launch: the next kernel starts after these writes are complete.
+// 2,213 -> 2,054. Neither triggers its dependents, and the forward's first kernel (k_embed) is launched without
+// the programmatic attribute, so that it starts after these writes are complete and visible.
 __global__ void __launch_bounds__(256) k_copy_words(const WordCopies w) {
   for (int c = 0; c < w.n_copies; ++c)
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < w.n[c]; i += gridDim.x * blockDim.x) w.dst[c][i] = w.src[c][i];

@@ -74,8 +74,9 @@ JF_DEV void jf_tl_record(unsigned kid, uint64_t t0, uint64_t t1) {
 #endif
 
 // ------------------------------------------------------------------------------------------
-// Programmatic dependent launch. Every kernel of the chain calls pdl_wait() before it reads
-// anything an earlier kernel wrote (and before it exits), so completion stays transitive.
+// Programmatic dependent launch. Every kernel of the chain but the forward's first (k_embed, a full
+// boundary) calls pdl_wait() before it reads anything an earlier kernel of the chain wrote (and before it
+// exits), so completion stays transitive.
 // ------------------------------------------------------------------------------------------
 JF_DEV void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 JF_DEV void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }

@@ -62,13 +62,17 @@ __global__ void k_rope_table(float2* tab, int n_pos, int half, double theta) {
   }
 }
 
-// x[r, :] = E[tok[r], :] (fp32 residual stream)
+// x[r, :] = E[tok[r], :] (fp32 residual stream). The first kernel of a forward, launched without the
+// programmatic attribute: it starts once everything before it on the stream is complete and visible, and the
+// forward's other kernels start after it. They may therefore read what was written before the forward (rows,
+// positions, the chain table, pages, weights) ahead of their own dependency wait; that wait alone would not
+// order such a read, as each kernel lets the next one in at its entry. The boundary costs nothing that was
+// hidden: what precedes a forward is a hand-over kernel of a few KB or another graph launch.
 template <typename T>
 __global__ void k_embed(const T* __restrict__ E, const int* __restrict__ tok, float* __restrict__ x, int d, int V,
                         int* err) {
   JF_TL_ENTRY();
   pdl_launch_dependents();
-  pdl_wait();
   JF_TL_WAITED();
   const int r = blockIdx.x;
   int t = tok[r];
@@ -371,9 +375,9 @@ __global__ void __launch_bounds__(128) k_qkv_finish(SplitPartials sp, const bf16
   if (job >= M * slots) return;
   const int m = job / slots, hs = job % slots;
   const bool rot = hs < Hq + Hkv;
-  // before the dependency wait: the bias (a weight), the row's position (written before this
-  // forward's kernels: by a host copy, or by the state machine after the previous forward) and its
-  // rotary coefficients (a table built at context creation)
+  // before the dependency wait: the bias (a weight), the row's position (written before this forward's
+  // first kernel began: by a hand-over kernel, or by the state machine after the previous forward) and
+  // its rotary coefficients (a table built at context creation)
   uint2 bw = make_uint2(0u, 0u);
   if (bias != nullptr) bw = *reinterpret_cast<const uint2*>(bias + (size_t)hs * 128 + lane * 4);
   float2 c0 = make_float2(1.f, 0.f), c1 = c0, c2 = c0, c3 = c0;
@@ -502,9 +506,9 @@ cudaError_t launch_rope_table(float2* tab, int n_pos, int half, double theta, cu
 
 cudaError_t launch_embed(const void* E, bool is_bf16, const int* tok, float* x, int rows, int d, int V, int* err,
                          cudaStream_t st) {
-  if (is_bf16)
-    return launch_pdl(k_embed<bf16>, dim3(rows), dim3(256), st, reinterpret_cast<const bf16*>(E), tok, x, d, V, err);
-  return launch_pdl(k_embed<float>, dim3(rows), dim3(256), st, reinterpret_cast<const float*>(E), tok, x, d, V, err);
+  if (is_bf16) k_embed<bf16><<<rows, 256, 0, st>>>(reinterpret_cast<const bf16*>(E), tok, x, d, V, err);
+  else k_embed<float><<<rows, 256, 0, st>>>(reinterpret_cast<const float*>(E), tok, x, d, V, err);
+  return cudaGetLastError();
 }
 
 template <int KS>

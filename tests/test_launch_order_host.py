@@ -1,0 +1,62 @@
+"""Which launches may start before the kernel ahead of them is complete, recorded on the host.
+
+The launch helpers of the forward's small kernels are compiled with a recorder in the place of
+cudaLaunchKernelEx and called without a GPU. Kernels of a forward read what was written before it (rows,
+positions, the chain table) ahead of their own dependency wait, and every kernel lets the next one in at its
+entry; so the first one, the embedding, must not be launched programmatically.
+"""
+import os
+import subprocess
+
+import pytest
+
+from paper_2512_14681_gb300 import build as B
+
+PRELUDE = r"""
+#include <cstdio>
+#include <cuda_runtime.h>
+struct Launch { int programmatic; dim3 grid; };
+static Launch g_last;
+static int g_launches;
+template <typename... E, typename... A>
+cudaError_t record_launch(const cudaLaunchConfig_t* c, void (*)(E...), A&&...) {
+  g_last = {0, c->gridDim};
+  for (unsigned i = 0; i < c->numAttrs; ++i)
+    if (c->attrs[i].id == cudaLaunchAttributeProgrammaticStreamSerialization)
+      g_last.programmatic = c->attrs[i].val.programmaticStreamSerializationAllowed;
+  ++g_launches;
+  return cudaSuccess;
+}
+#define cudaLaunchKernelEx record_launch
+"""
+
+
+def run_host(tmp_path, source, body):
+    """Output lines of `body` (a main) compiled behind csrc/`source` and the recorder."""
+    try:
+        nvcc = B.nvcc()
+    except RuntimeError:
+        pytest.skip("needs nvcc")
+    src = tmp_path / "host.cu"
+    src.write_text(PRELUDE + f'#include "{os.path.join(B.CSRC, source)}"\n' + body)
+    exe = tmp_path / "host"
+    r = subprocess.run([nvcc, *B.ARCH, "-std=c++17", "-O0", "-Xcicc", "-O0", "-Xptxas", "-O0", "--expt-relaxed-constexpr",
+                        "-I", B.CSRC, "-I", os.path.join(B.ROOT, "include"), str(src), "-o", str(exe)],
+                       capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr
+    return subprocess.run([str(exe)], capture_output=True, text=True, check=True, env=dict(os.environ, CUDA_VISIBLE_DEVICES="")).stdout.split()
+
+
+def test_the_first_kernel_of_a_forward_is_a_full_boundary(tmp_path):
+    out = run_host(tmp_path, "jf_elementwise.cu", r"""
+int main() {
+  for (int bf16 = 0; bf16 < 2; ++bf16) {
+    g_launches = g_last.programmatic = 0;
+    jf::launch_embed(nullptr, bf16, nullptr, nullptr, 4, 256, 512, nullptr, 0);
+    std::printf("%d ", g_launches ? g_last.programmatic : 0);
+    jf::launch_rmsnorm(nullptr, nullptr, nullptr, bf16, 4, 256, 1e-6f, nullptr, 0, 0);
+    std::printf("%d ", g_last.programmatic);
+  }
+}
+""")
+    assert out == ["0", "1", "0", "1"]  # embedding, norm; fp32, bf16
