@@ -61,7 +61,8 @@ JF_DEV uint8_t* align1024(uint8_t* p) {
 
 // ---------------------------------------------------------------------------------------------
 // Greedy argmax. Logits are compared through keys that preserve their order as unsigned integers (-0
-// counts as +0, NaN as the lowest, key 0). Every CTA keeps a running entry (best key, its lowest index,
+// counts as +0, NaN as the lowest, key 0). A row without a number gets the index kAmNoIndex, which no
+// vocabulary holds: the callers see it, and the next forward's embedding reports it. Every CTA keeps a running entry (best key, its lowest index,
 // runner-up key) of every row over the vocabulary tiles it takes: in shared memory for up to
 // kAmTableRows rows, otherwise in its global slot; k_argmax_finish merges the CTAs' slots. The merge is
 // associative and commutative, so the result does not depend on which CTA took which tile. With
@@ -73,7 +74,10 @@ JF_DEV uint32_t am_key(float v) {
   const uint32_t u = __float_as_uint(v + 0.0f);
   return v != v ? 0u : ((u & 0x80000000u) ? ~u : (u | 0x80000000u));
 }
-JF_DEV float am_value(uint32_t key) { return __uint_as_float((key & 0x80000000u) ? key ^ 0x80000000u : ~key); }
+// (no number under a key of 0: -infinity)
+JF_DEV float am_value(uint32_t key) {
+  return key == 0u ? -INFINITY : __uint_as_float((key & 0x80000000u) ? key ^ 0x80000000u : ~key);
+}
 JF_DEV void am_merge(uint32_t& b1, uint32_t& bi, uint32_t& b2, uint32_t o1, uint32_t oi, uint32_t o2) {
   if (o1 > b1 || (o1 == b1 && oi < bi)) {
     b2 = b1 > o2 ? b1 : o2;
@@ -137,7 +141,7 @@ __global__ void __launch_bounds__(128) k_argmax_finish(const uint32_t* k1, const
     const uint32_t best = __reduce_min_sync(0xffffffffu, b1 == top ? bi : 0xffffffffu);
     const uint32_t second = __reduce_max_sync(0xffffffffu, (b1 == top && bi == best) ? b2 : b1);
     if (lane == 0) {
-      out[m] = (int)best;
+      out[m] = (int)(top == 0u ? kAmNoIndex : best);
       if (top2) {
         top2[2 * m] = am_value(top);
         top2[2 * m + 1] = am_value(second);
