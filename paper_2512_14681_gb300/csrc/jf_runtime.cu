@@ -914,7 +914,7 @@ jf_status generate_impl(jf_ctx* c, int n_seqs, const int32_t* const* h_prompts, 
                      c->res_host, c->err, c->st));
   c->launches += 1;
   CK(cudaStreamSynchronize(c->st));
-  jf_status s = check_err_word(c, c->res_host->err);
+  jf_status s = take_err(c, c->res_host->err);
   if (s != JF_OK) return s;
   int M = c->res_host->next_M;
   int iters = 0;
@@ -937,7 +937,7 @@ jf_status generate_impl(jf_ctx* c, int n_seqs, const int32_t* const* h_prompts, 
     if (c->profiling) accumulate_profile(c, gr);
     rows_log.push_back(M);
     ++iters;
-    if ((s = check_err_word(c, c->res_host->err)) != JF_OK) return s;
+    if ((s = take_err(c, c->res_host->err)) != JF_OK) return s;
     done = c->res_host->all_done != 0;
     M = c->res_host->next_M;
     // every forward commits a token or a prefill chunk of some sequence

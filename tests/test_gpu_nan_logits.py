@@ -1,8 +1,8 @@
 """Rows whose logits hold no number (weights that overflowed) are reported, not decoded as token 0.
 
 Infinite weights make every logit NaN. The argmax then is 0x7fffffff with -infinity for the best two
-logits, prefill and the forward show it to the caller, and a generation ends with JF_EDEVICE at the forward that
-would read that token.
+logits, prefill and the forward show it to the caller, a generation ends with JF_EDEVICE at the forward that
+would read that token, and the context works again with finite weights.
 """
 import math
 
@@ -37,5 +37,9 @@ def test_rows_without_a_number_are_reported(bf16):
         with pytest.raises(JfError) as e:
             ctx.generate([prompt], Gen(block_size=4, max_new=8))
         assert e.value.status == JF_EDEVICE
+        # reading the error cleared it
+        ctx.init_random_weights(I.WEIGHT_SEED, I.WEIGHT_STD)
+        ctx.truncate(0, 0)
+        assert 0 <= ctx.prefill(0, prompt) < shape.vocab
     finally:
         ctx.close()
