@@ -109,6 +109,9 @@ struct GemmParams {
   int* tile_counter;   // [m_tiles*n_tiles], zero between launches
   int* err;
   unsigned long long wait_ns;  // limit of each bounded wait
+  // bf16 path: programmatic launch. Only where W was complete before the kernels that may still run began (a
+  // context's weights): its first tiles are requested ahead of the dependency wait.
+  bool overlap;
   GemmEpi epi;
 };
 
