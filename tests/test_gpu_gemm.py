@@ -95,3 +95,32 @@ def test_gemm_f32_matches_oracle():
     assert int(err.item()) == 0
     ref = O.linear(X.astype(np.float64), W.astype(np.float64))
     assert np.abs(Y.cpu().numpy() - ref).max() < 1e-4
+
+
+@pytest.mark.parametrize("first,second", [((300, 4), (32, 4)), ((32, 4), (300, 4)), ((200, 8), (64, 2)), ((600, 2), (600, 3))])
+def test_gemm_bf16_shapes_share_a_workspace(first, second):
+    """Calls of two shapes through one workspace zeroed once: the tickets of the second one lie where the
+    first one's partial tiles may be. Every element of Y is written, with the bits of a call of its own."""
+    torch = need_gpu()
+    import ctypes
+
+    from paper_2512_14681_gb300 import _lib as J
+    from paper_2512_14681_gb300.jacobi import op_gemm
+
+    lib, N, K = J.load(), 640, 2048
+    W = _bf16(torch, I.random_array((N, K), seed=21, scale=0.5))
+    nb = ctypes.c_size_t()
+    need = 0
+    for M, splits in (first, second):
+        assert lib.jf_op_gemm_workspace_bytes(N, K, M, splits, ctypes.byref(nb)) == J.JF_OK
+        need = max(need, nb.value)
+    ws, err = torch.zeros(need, dtype=torch.uint8, device="cuda"), torch.zeros(1, dtype=torch.int32, device="cuda")
+    for M, splits in (first, second):
+        X = _bf16(torch, I.random_array((M, K), seed=M, scale=0.5))
+        Y = torch.full((M, N), float("nan"), device="cuda")
+        assert lib.jf_op_gemm(J.JF_BF16, W.data_ptr(), X.data_ptr(), Y.data_ptr(), N, K, M, splits, ws.data_ptr(), need,
+                              err.data_ptr(), torch.cuda.current_stream().cuda_stream) == J.JF_OK
+        alone, _, _ = op_gemm(W, X, k_splits=splits)
+        torch.cuda.synchronize()
+        assert int(err.item()) == 0
+        assert torch.equal(Y, alone)
