@@ -145,18 +145,6 @@ JF_DEV uint32_t tc_swz(int r, int c16) {
   return (uint32_t)((c16 >> 3) * TC_BLK + r * 128 + (((c16 & 7) ^ (r & 7)) << 4));
 }
 
-// Barrier of the softmax warps (barrier 0 is __syncthreads); true when every thread's `ok` is.
-JF_DEV bool softmax_sync_and(bool ok) {
-  uint32_t r;
-  asm volatile(
-      "{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, %1, 0;\n\t"
-      "barrier.cta.red.and.pred q, 1, 256, p;\n\tselp.u32 %0, 1, 0, q;\n\t}"
-      : "=r"(r)
-      : "r"((int)ok)
-      : "memory");
-  return r != 0;
-}
-
 // The steps of one CTA: the chunks of its lanes j, j + n_ctas, ..., lane after lane.
 struct Cursor {
   int ln, chunk;
@@ -416,7 +404,7 @@ __global__ void __launch_bounds__(ATT_THREADS, 1)
       tc_commit(smem_u32(&b_kfree[stage]));
     };
     if (n_steps > 0) {
-      ok = mbar_wait_bounded(smem_u32(&b_q), 0u, a.wait_ns);
+      ok = __all_sync(0xffffffffu, mbar_wait_bounded(smem_u32(&b_q), 0u, a.wait_ns));
       Cursor c{j, j};
       int stage = 0;  // K stage and phase of step t+2
       uint32_t parity = 0;
@@ -496,7 +484,7 @@ __global__ void __launch_bounds__(ATT_THREADS, 1)
     // unit, O stored as [dim / 4][row][4] (a warp writes 512 contiguous bytes for 4 dimensions).
     auto finish_lane = [&](int ln, int t_end, float m) {
       if (!mbar_wait_bounded(smem_u32(&b_o[t_end & 1]), (uint32_t)(t_end >> 1) & 1u, a.wait_ns)) {
-        if (tid == 0) jf_set_error(a.err, JF_DERR_TIMEOUT_MMA);
+        jf_set_error(a.err, JF_DERR_TIMEOUT_MMA);
         ok = false;
       }
       tc_fence_after();
@@ -540,7 +528,7 @@ __global__ void __launch_bounds__(ATT_THREADS, 1)
     for (int t = 0; t <= n_steps; ++t) {
       const bool step = t < n_steps;  // after the last step only the last lane is finished
       if (step && !mbar_wait_bounded(smem_u32(&b_s[t & 1]), (uint32_t)(t >> 1) & 1u, a.wait_ns)) {
-        if (tid == 0) jf_set_error(a.err, JF_DERR_TIMEOUT_MMA);
+        jf_set_error(a.err, JF_DERR_TIMEOUT_MMA);
         ok = false;
       }
       tc_fence_after();
@@ -577,7 +565,7 @@ __global__ void __launch_bounds__(ATT_THREADS, 1)
         }
         red_max[t & 1][half][r] = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])) * scale;
       }
-      ok = softmax_sync_and(ok);
+      ok = sync_and<1, SOFTMAX_THREADS>(ok);  // (barrier 0 is __syncthreads)
       if (!ok) break;
       bool raise = false;
       float mc = -INFINITY;
@@ -588,7 +576,7 @@ __global__ void __launch_bounds__(ATT_THREADS, 1)
       if (!first && __any_sync(0xffffffffu, raise)) {
         // the same for both column halves of the warp's rows; alpha = 1 leaves a row as it is
         if (!mbar_wait_bounded(smem_u32(&b_o[(t - 1) & 1]), (uint32_t)((t - 1) >> 1) & 1u, a.wait_ns)) {
-          if (lane == 0) jf_set_error(a.err, JF_DERR_TIMEOUT_MMA);
+          jf_set_error(a.err, JF_DERR_TIMEOUT_MMA);
           ok = false;
         }
         tc_fence_after();

@@ -132,6 +132,20 @@ JF_DEV bool mbar_wait_bounded(uint32_t bar, uint32_t parity, uint64_t limit_ns) 
   }
 }
 
+// Barrier ID of N threads (whole warps, in any convergence); true when every thread's `ok` is. A wait's outcome
+// may differ from thread to thread when its phase completes near the limit: threads that meet at barriers or in
+// warp-wide instructions afterwards agree on it first, and leave together.
+template <int ID, int N>
+JF_DEV bool sync_and(bool ok) {
+  uint32_t r;
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, %1, 0;\n\t"
+      "barrier.cta.red.and.pred q, %2, %3, p;\n\tselp.u32 %0, 1, 0, q;\n\t}"
+      : "=r"(r)
+      : "r"((int)ok), "n"(ID), "n"(N)
+      : "memory");
+  return r != 0;
+}
 
 // ------------------------------------------------------------------------------------------
 // Thread-block clusters: ranks, cluster-wide barrier

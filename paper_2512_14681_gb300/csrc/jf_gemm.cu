@@ -586,7 +586,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
       for (int u = first_unit; u < total_units && ok; u += unit_step, ++i) {
         const Unit w = unit_of(p, u);
         const int acc = i & 1;
-        if (i >= 2 && !mbar_wait_bounded(tempty0 + 8 * acc, (uint32_t)((i >> 1) - 1) & 1u, p.wait_ns)) {
+        if (i >= 2 && !__all_sync(0xffffffffu, mbar_wait_bounded(tempty0 + 8 * acc, (uint32_t)((i >> 1) - 1) & 1u, p.wait_ns))) {
           if (lane == 0) jf_set_error(p.err, JF_DERR_TIMEOUT_EPI);
           break;
         }
@@ -652,8 +652,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     for (int u = first_unit; u < total_units; u += unit_step, ++i) {
       const Unit w = unit_of(p, u);
       const int acc = i & 1;
-      if (!mbar_wait_bounded(tfull0 + 8 * acc, (uint32_t)(i >> 1) & 1u, p.wait_ns)) {
-        jf_set_error(p.err, JF_DERR_TIMEOUT_EPI);
+      // agreed on by all epilogue threads: they share barriers below
+      const bool ready = mbar_wait_bounded(tfull0 + 8 * acc, (uint32_t)(i >> 1) & 1u, p.wait_ns);
+      if (!sync_and<3, 128 * EPI_HALVES>(ready)) {
+        if (!ready) jf_set_error(p.err, JF_DERR_TIMEOUT_EPI);
         break;
       }
       tc_fence_after();
