@@ -235,6 +235,7 @@ JF_DEV bool load_steps(const AttnParams& a, const AttnUnit& u, int j, int n_ctas
         cp_async_commit();
         cp_async_wait<0>();
         fence_proxy_async_smem();  // this thread's cp.async writes -> tensor-core operand reads
+        __syncwarp();              // every lane's, before lane 0's arrival
       }
     }
     const uint32_t total = __reduce_add_sync(0xffffffffu, bytes);

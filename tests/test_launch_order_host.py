@@ -3,7 +3,8 @@
 The launch helpers of the forward's small kernels are compiled with a recorder in the place of
 cudaLaunchKernelEx and called without a GPU. Kernels of a forward read what was written before it (rows,
 positions, the chain table) ahead of their own dependency wait, and every kernel lets the next one in at its
-entry; so the first one, the embedding, must not be launched programmatically.
+entry; so the first one, the embedding, must not be launched programmatically. The last test reads the source
+for an order that no run can show.
 """
 import os
 import subprocess
@@ -60,3 +61,12 @@ int main() {
 }
 """)
     assert out == ["0", "1", "0", "1"]  # embedding, norm; fp32, bf16
+
+
+def test_copied_rows_are_ordered_before_the_arrival():
+    """The attention's loaders: what 32 lanes copied is published by lane 0's arrival, so the lanes meet between."""
+    text = open(os.path.join(B.CSRC, "jf_attention.cu")).read()
+    text = text[text.index("JF_DEV bool load_steps("):]
+    copied, arrival = text.index("cp_async_wait<0>();"), text.index("mbar_arrive_expect_tx(")
+    fence = text.index("fence_proxy_async_smem();", copied)
+    assert copied < fence < text.index("__syncwarp();", fence) < arrival
