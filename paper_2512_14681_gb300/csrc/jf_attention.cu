@@ -194,6 +194,7 @@ JF_DEV bool load_steps(const AttnParams& a, const AttnUnit& u, int j, int n_ctas
   c = Cursor{j, j};
   int id_next = n_steps > 0 ? page_id(c.chunk) : -1, stage = 0;
   uint32_t parity = 1u;  // of the stage's previous use
+  bool done = true;
   pdl_wait();  // in-flight keys come from the QKV projection
 #pragma unroll 1
   for (int t = 0; t < n_steps; ++t) {
@@ -202,7 +203,11 @@ JF_DEV bool load_steps(const AttnParams& a, const AttnUnit& u, int j, int n_ctas
     if (t + 1 < n_steps) id_next = page_id(c.chunk);
     if (t >= n_stages) {
       const bool ok = mbar_wait_bounded(smem_u32(&freed[stage]), parity, a.wait_ns);
-      if (!__all_sync(0xffffffffu, ok)) return false;
+      if (!__all_sync(0xffffffffu, ok)) {
+        n_steps = t;
+        done = false;
+        break;
+      }
       copy_cached(chunk, id, stage);
     }
     const uint32_t dst = stages + (uint32_t)(stage * TC_OPND), bar = smem_u32(&full[stage]);
@@ -245,7 +250,10 @@ JF_DEV bool load_steps(const AttnParams& a, const AttnUnit& u, int j, int n_ctas
       parity ^= 1u;
     }
   }
-  return true;
+  // every copy has landed before the CTA may leave, also after a wait that gave up
+  for (int t = n_steps > n_stages ? n_steps - n_stages : 0; t < n_steps; ++t)
+    if (!mbar_wait_bounded(smem_u32(&full[t % n_stages]), (uint32_t)(t / n_stages) & 1u, a.wait_ns)) break;
+  return done;
 }
 
 // Fold of rows rb*16 .. rb*16+15 of unit ui over its 8 lane states in lane order (thread: row
@@ -317,8 +325,8 @@ __global__ void __launch_bounds__(ATT_THREADS, 1)
   uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(sm_raw) + 1023) & ~uintptr_t(1023));
   const uint32_t sQ = smem_u32(sm), sK = smem_u32(sm + TC_OFF_K), sV = smem_u32(sm + TC_OFF_V);
   // per K stage: loaded / read; per V stage: loaded; per parity of the step: S ready, P ready, P V done
-  // (which also frees the V stage); Q loaded
-  __shared__ __align__(8) uint64_t b_kfull[K_STAGES], b_kfree[K_STAGES], b_vfull[V_STAGES], b_s[2], b_p[2], b_o[2], b_q;
+  // (which also frees the V stage); Q loaded; all MMAs done
+  __shared__ __align__(8) uint64_t b_kfull[K_STAGES], b_kfree[K_STAGES], b_vfull[V_STAGES], b_s[2], b_p[2], b_o[2], b_q, b_all;
   __shared__ uint32_t tmem_slot;
   __shared__ AttnUnit s_unit;
   __shared__ float red_max[2][2][kAttnQRows];  // [step parity][column half][row]
@@ -343,6 +351,7 @@ __global__ void __launch_bounds__(ATT_THREADS, 1)
       mbar_init(smem_u32(&b_p[i]), SOFTMAX_THREADS / 32);
       mbar_init(smem_u32(&b_o[i]), 1);
     }
+    mbar_init(smem_u32(&b_all), 1);
     mbar_init(smem_u32(&b_q), by_token ? 1 : SOFTMAX_THREADS / 32);
     fence_mbar_init();
   }
@@ -448,6 +457,11 @@ __global__ void __launch_bounds__(ATT_THREADS, 1)
         }
       }
       if (!ok && lane == 0) jf_set_error(a.err, JF_DERR_TIMEOUT_MMA);
+      // Q has landed and every MMA is complete before the CTA may leave, also after a wait that gave up
+      if (elect_one()) tc_commit(smem_u32(&b_all));
+      __syncwarp();
+      mbar_wait_bounded(smem_u32(&b_q), 0u, a.wait_ns);
+      mbar_wait_bounded(smem_u32(&b_all), 0u, a.wait_ns);
     }
     __syncwarp();
   } else {

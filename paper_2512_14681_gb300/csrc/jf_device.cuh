@@ -298,6 +298,11 @@ JF_DEV void tc_commit_pair(uint32_t bar) {
       : "memory");
 }
 
+// The same arrival on rank 0's mbarrier alone.
+JF_DEV void tc_commit_pair_local(uint32_t bar) {
+  asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+}
+
 // Load 16 consecutive fp32 columns of this warp's 32 TMEM lanes (lane = thread).
 JF_DEV void tmem_ld16(uint32_t taddr, float (&v)[16]) {
   uint32_t r[16];

@@ -422,7 +422,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
   uint64_t* bars = reinterpret_cast<uint64_t*>(reinterpret_cast<uint8_t*>(xs) + EPI_STAGE_BYTES);
   const uint32_t idle = smem_u32(bars + 2 * D + 4);  // never completes: a wait for its odd phase passes
   const uint32_t sink = smem_u32(bars + 2 * D + 5);  // nobody waits for it
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * D + 6);
+  const uint32_t all_done = smem_u32(bars + 2 * D + 6);  // every MMA of this CTA (of the pair, in rank 0)
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * D + 7);
   int* sflag = reinterpret_cast<int*>(tmem_slot + 1);
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -481,6 +482,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     }
     mbar_init(idle, 1);
     mbar_init(sink, 1);
+    mbar_init(all_done, 1);
     fence_mbar_init();
     tma_prefetch_desc(&tmA);
     tma_prefetch_desc(&tmB);
@@ -531,7 +533,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     u = __shfl_sync(0xffffffffu, u, pre - 1);
     int kb = __shfl_sync(0xffffffffu, kb0, pre - 1) + 2;
     Unit w = unit_of(p, u);
-    int d = pre == D ? 0 : pre;
+    int d = pre == D ? 0 : pre, issued = pre;
     uint32_t parity = 0u;
 #pragma unroll 1
     for (int q = -1; q <= 0 || pre + q < total_iters; ++q) {
@@ -559,6 +561,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
       }
       __syncwarp();
       if (on) {
+        ++issued;
         kb += 2;
         if (++d == D) {
           d = 0;
@@ -566,6 +569,11 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         }
       }
     }
+    // Every copy has landed before the CTA may leave, also after a wait that gave up (a pair's complete on rank
+    // 0's barriers; when a wait gives up here too, the copies have had its limit to land).
+    if (rank == 0)
+      for (int q = issued > D ? issued - D : 0; q < issued; ++q)
+        if (!mbar_wait_bounded(full0 + 8 * (q % D), (uint32_t)(q / D) & 1u, p.wait_ns)) break;
     if constexpr (PAIR) {  // rank 0's last arrivals on this CTA's barriers, before it may leave
       for (int q = total_iters > D ? total_iters - D : 0; q < total_iters; ++q)
         if (!mbar_wait_bounded(empty0 + 8 * (q % D), (uint32_t)(q / D) & 1u, p.wait_ns)) break;
@@ -631,6 +639,13 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
           }
         }
       }
+      // every MMA is complete before the tensor memory is given back, also after a wait that gave up
+      if (elect_one()) {
+        if constexpr (PAIR) tc_commit_pair_local(all_done);
+        else tc_commit(all_done);
+      }
+      __syncwarp();
+      mbar_wait_bounded(all_done, 0u, p.wait_ns);
     }
     __syncwarp();
   } else {
