@@ -766,7 +766,7 @@ cudaError_t launch_commit(const CommitInfo* commit, int n_seqs, int rows, int L,
                           void* k_pages, void* v_pages, const int* page_table, int pages_per_seq, int n_pages,
                           int max_rows, int Hkv, int hd, int elem_bytes, int* seq_len, int* err, cudaStream_t st) {
   cudaLaunchAttribute at[1];
-  // four pieces a thread when every row in flight is accepted; more if that is over 64 blocks
+  // four pieces a thread when a sequence commits all it can; more if that is over 64 blocks
   const long long pieces = (long long)rows * Hkv * hd * elem_bytes / 16;
   const int z = (int)(pieces <= 1024 ? 1 : (pieces + 1023) / 1024 < 64 ? (pieces + 1023) / 1024 : 64);
   cudaLaunchConfig_t cfg = pdl_cfg(dim3(L, n_seqs, z), dim3(256), 0, st, at);

@@ -31,7 +31,7 @@ struct GenCfg {
   // forward j on, prefill_chunk rows per forward), prompt offset in `prompts`, prompt length.
   const int* seq_params;
   const int* prompts;     // prompts of the sequences that join later (device)
-  int prefill_chunk;
+  int prefill_chunk;      // 0: none does
 };
 constexpr int kSeqParams = 5;
 enum SeqParam : int { SP_N = 0, SP_SSPAWN, SP_JOIN, SP_POFF, SP_PLEN };
@@ -127,7 +127,13 @@ cudaError_t launch_traj_noisy(const int* traj, int n_rec, int R, int seq, const 
                               int n_blocks, int* noisy, int* point, cudaStream_t st);
 cudaError_t launch_step_accept(const StepBlocks* sb, const int* tok, const int* gpred, int* committed,
                                CommitInfo* commit, StepResult* res, int* err, cudaStream_t st);
-// rows: rows in flight of the forward, an upper bound of what one sequence commits
+// Rows that one sequence can commit in an iteration of M rows in flight: a block, or a chunk of its prompt where
+// sequences join late (prefill_chunk is 0 otherwise).
+inline int commit_rows(const GenCfg& g, int M) {
+  const int most = g.n > g.prefill_chunk ? g.n : g.prefill_chunk;
+  return most < M ? most : M;
+}
+// rows: about what one sequence commits at the most (sizes the grid)
 cudaError_t launch_commit(const CommitInfo* commit, int n_seqs, int rows, int L, const void* k_inf, const void* v_inf,
                           void* k_pages, void* v_pages, const int* page_table, int pages_per_seq, int n_pages,
                           int max_rows, int Hkv, int hd, int elem_bytes, int* seq_len, int* err, cudaStream_t st);

@@ -672,7 +672,7 @@ cudaError_t enqueue_iteration(jf_ctx* c, const GenCfg& g, int M, int n_seqs) {
   prof_end(c);
   if (e != cudaSuccess) return e;
   prof_begin(c, PC_OTHER);
-  e = launch_commit(c->commit, n_seqs, M, D.L, c->k_inf, c->v_inf, c->k_pages, c->v_pages, c->page_table, D.pps,
+  e = launch_commit(c->commit, n_seqs, commit_rows(g, M), D.L, c->k_inf, c->v_inf, c->k_pages, c->v_pages, c->page_table, D.pps,
                     D.n_pages, D.R, D.Hkv, D.hd, D.es, c->seq_len, c->err, c->st);
   prof_end(c);
   if (e != cudaSuccess) return e;
@@ -903,7 +903,7 @@ jf_status generate_impl(jf_ctx* c, int n_seqs, const int32_t* const* h_prompts, 
   g.out_tokens = c->gen_out; g.iter_log = c->gen_log; g.max_iters = D.max_ctx;
   g.seq_params = c->gen_seqp;
   g.prompts = c->gen_prompt;
-  g.prefill_chunk = chunk;
+  g.prefill_chunk = loff > 0 ? chunk : 0;
   if (want_traj) {
     g.traj = stats->traj;
     g.traj_cap = stats->traj_cap;
@@ -1453,7 +1453,7 @@ jf_status jf_jacobi_step(jf_ctx* c, int seq, int n_blocks, const jf_block* block
   c->chains_bound = nch;
   CK(enqueue_forward(c, total, LM_ARGMAX));
   CK(launch_step_accept(c->sb_dev, c->tok, c->gpred, c->committed_dev, c->commit, c->sres_dev, c->err, c->st));
-  CK(launch_commit(c->commit + seq, 1, total, D.L, c->k_inf, c->v_inf, c->k_pages, c->v_pages,
+  CK(launch_commit(c->commit + seq, 1, max_len, D.L, c->k_inf, c->v_inf, c->k_pages, c->v_pages,
                    c->page_table + (size_t)seq * D.pps, D.pps, D.n_pages, D.R, D.Hkv, D.hd, D.es, c->seq_len + seq,
                    c->err, c->st));
   StepResult r;

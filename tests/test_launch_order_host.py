@@ -1,4 +1,4 @@
-"""Which launches may start before the kernel ahead of them is complete, recorded on the host.
+"""Launch attributes and grids of the forward's small kernels, recorded on the host.
 
 The launch helpers of the forward's small kernels are compiled with a recorder in the place of
 cudaLaunchKernelEx and called without a GPU. Kernels of a forward read what was written before it (rows,
@@ -61,6 +61,25 @@ int main() {
 }
 """)
     assert out == ["0", "1", "0", "1"]  # embedding, norm; fp32, bf16
+
+
+def test_the_commit_grid_follows_what_one_sequence_commits(tmp_path):
+    """16 sequences of 32 rows, 28 layers of 4 KV heads: 2,048 pieces of 16 bytes a sequence, two blocks; where
+    prompts join in chunks of 64 rows, four. One sequence of 4 rows: one block."""
+    out = run_host(tmp_path, "jf_decode.cu", r"""
+int main() {
+  jf::GenCfg g = {};
+  const int cfg[3][4] = {{32, 0, 512, 16}, {32, 64, 512, 16}, {32, 0, 4, 1}};  // block, chunk, rows in flight, sequences
+  for (auto& c : cfg) {
+    g.n = c[0];
+    g.prefill_chunk = c[1];
+    jf::launch_commit(nullptr, c[3], jf::commit_rows(g, c[2]), 28, nullptr, nullptr, nullptr, nullptr, nullptr, 64, 64, 512, 4,
+                      128, 2, nullptr, nullptr, 0);
+    std::printf("%u,%u,%u ", g_last.grid.x, g_last.grid.y, g_last.grid.z);
+  }
+}
+""")
+    assert out == ["28,16,2", "28,16,4", "28,1,1"]
 
 
 def test_copied_rows_are_ordered_before_the_arrival():
