@@ -67,7 +67,7 @@ typedef struct {
 
 /* Capacity. max_rows: in-flight rows per forward (K*n + candidates, or a prefill chunk);
  * max_ctx: positions per sequence (KV pages of 16 tokens are reserved for it; at most 130944
- *   for JF_BF16 models, whose attention stages a sequence's page ids in shared memory);
+ *   for JF_BF16 models);
  * logits_rows: rows jf_forward_logits() may return (0 = that call is unavailable);
  * page_size: tokens per KV page, 0 or 16 (the only size the kernels support; others are
  *   JF_EUNSUPPORTED);

@@ -1,7 +1,7 @@
 // Launch form of the split-KV attention (host side; no CUDA types, so that the rule compiles and is
 // tested on the host alone).
 //
-// A unit (chain, KV head, tile of 128 query rows) has 8 key lanes, spread over 8, 4, 2 or 1 CTAs (one
+// A unit (chain, KV head, tile of up to 128 query rows) has 8 key lanes, spread over 8, 4, 2 or 1 CTAs (one
 // cluster; one CTA per SM). max_clusters[i] clusters of 2^i CTAs are resident at once (152, 76, 36, 15
 // on a GB300). Wide clusters shorten a unit, narrow ones fit more units at once and fold less through
 // memory. Every form computes the same lane states and folds them in the same order, so the choice
@@ -20,13 +20,10 @@ inline int attn_units_estimate(int M, int chains, int units_bound, int Hkv, int 
   return est < units_bound ? (int)est : units_bound;
 }
 
-// true: clusters of `max_clusters` at once need no more waves of units than `lanes` independent places
-// per unit on `num_sms` of them do.
-inline bool attn_use_clusters(int units, int lanes, int max_clusters, int num_sms) {
-  const int mc = max_clusters > 0 ? max_clusters : 1;
-  const int waves_clustered = (units + mc - 1) / mc;
-  const int waves_unclustered = (int)(((long long)units * lanes + num_sms - 1) / num_sms);
-  return waves_clustered <= waves_unclustered;
+// Waves of `units` units with `at_once` of them resident at a time (none known: one).
+inline int attn_waves(int units, int at_once) {
+  const int n = at_once > 0 ? at_once : 1;
+  return (units + n - 1) / n;
 }
 
 // CTAs per unit: the widest clusters that need no more waves than the next narrower ones. Past one wave
@@ -37,9 +34,8 @@ inline bool attn_use_clusters(int units, int lanes, int max_clusters, int num_sm
 // 331 / 309.
 inline int attn_ctas_per_unit(int units, const int (&max_clusters)[4]) {
   for (int i = 3; i > 0; --i)
-    if (attn_use_clusters(units, 1, max_clusters[i], max_clusters[i - 1])) return 1 << i;
-  const int w1 = (units + max_clusters[0] - 1) / max_clusters[0], w2 = (units + max_clusters[1] - 1) / max_clusters[1];
-  return w2 * 5 < w1 * 9 ? 2 : 1;
+    if (attn_waves(units, max_clusters[i]) <= attn_waves(units, max_clusters[i - 1])) return 1 << i;
+  return attn_waves(units, max_clusters[1]) * 5 < attn_waves(units, max_clusters[0]) * 9 ? 2 : 1;
 }
 
 }  // namespace jf

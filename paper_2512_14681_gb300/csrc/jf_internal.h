@@ -33,8 +33,8 @@ constexpr int kAttnQRows = 128;   // most (token, head) query rows per attention
 // Query rows of a unit's tile with G query heads per KV head: as many whole tokens as fit, so that one
 // TMA box (G heads x tokens) loads them; a group wider than the tile is cut anywhere.
 __host__ __device__ constexpr int attn_tile_rows(int G) { return G <= kAttnQRows ? kAttnQRows / G * G : kAttnQRows; }
-constexpr int kAttnLanes = 8;     // chunk lanes per unit (c mod 8); one CTA of an 8-CTA cluster each
-constexpr int kAttnLaneChunks = 128;  // chunks per lane the kernel can stage page ids for
+constexpr int kAttnLanes = 8;     // chunk lanes per unit (c mod 8), spread over the unit's 8, 4, 2 or 1 CTAs
+constexpr int kAttnLaneChunks = 128;  // most chunks per lane: the context limit of the interface
 constexpr int kAttnMaxCtx = kAttnChunk * kAttnLanes * kAttnLaneChunks;  // 131072 key positions
 constexpr int kAttnXchgFloats = kAttnQRows * 128 + 2 * kAttnQRows;   // one lane state: O (hd 128), m, l
 constexpr int kMaxSeqs = 64;

@@ -160,7 +160,7 @@ jf_status make_dims(const jf_model_config* m, const jf_runtime_config* rt, Dims*
     return JF_EINVAL;
   }
   if (m->dtype == JF_BF16 && rt->max_ctx > kAttnMaxCtx - kAttnChunk) {
-    *why = "max_ctx above the bf16 attention's page-id staging capacity (130944 positions)";
+    *why = "max_ctx above the bf16 attention's limit (130944 positions)";
     return JF_EINVAL;
   }
   D->L = m->n_layers; D->d = m->d_model; D->Hq = m->n_heads; D->Hkv = m->n_kv_heads; D->hd = m->head_dim;

@@ -1,11 +1,9 @@
-"""The attention's launch-form rule (csrc/jf_attn_form.h), compiled for the host and run without a GPU.
+"""The attention's launch rule (csrc/jf_attn_form.h), from rows and chains to CTAs per unit, on the host.
 
-A unit (chain, KV head, 128-row query tile) runs on 8 CTAs; as an 8-CTA cluster only 15 fit on a
-GB300's 152 SMs at once (cudaOccupancyMaxActiveClusters, measured), as independent CTAs all 152 do.
-The rule takes the clustered form unless the unclustered one needs fewer waves of units. The cases
-below are the 7B shape (4 KV heads, 7 query heads each) at the sweep's measured points, where the
-form it picks was the faster one, and the small model's 256-row window that the GPU test of the
-unclustered form relies on.
+A unit (chain, KV head, tile of up to 128 query rows of whole tokens) runs on a cluster of 8, 4 or 2 CTAs or on
+one. The cases are the 7B shape (4 KV heads, 7 query heads each: tiles of 126 rows) at the row and chain
+counts of the window sweep, and the small model (2 KV heads, 4 query heads each: tiles of 128) at those of the
+GPU tests that compare its forms. A GB300 holds 152 single CTAs, 76 pairs, 36 clusters of 4 and 15 of 8.
 """
 import os
 import shutil
@@ -22,38 +20,41 @@ PROGRAM = r"""
 
 #define CHECK(c) do { if (!(c)) { std::printf("FAIL line %d: %s\n", __LINE__, #c); return 1; } } while (0)
 
-static bool clustered(int M, int chains, int Hkv, int G) {
-  const int bound = Hkv * ((M * G + 127) / 128 + chains);
-  const int units = jf::attn_units_estimate(M, chains, bound, Hkv, G, 128);
-  return jf::attn_use_clusters(units, 8, 15, 152);
+static int ctas(int M, int chains, int Hkv, int G) {
+  const int tile = 128 / G * G, bound = Hkv * ((M * G + tile - 1) / tile + chains);
+  const int mc[4] = {152, 76, 36, 15};
+  return jf::attn_ctas_per_unit(jf::attn_units_estimate(M, chains, bound, Hkv, G, tile), mc);
 }
 
 int main() {
-  // unit estimates: rows spread over the chains, whole 128-row tiles per chain and KV head
-  CHECK(jf::attn_units_estimate(32, 1, 12, 4, 7, 128) == 8);      // 224 query rows: 2 tiles x 4 heads
-  CHECK(jf::attn_units_estimate(64, 4, 32, 4, 7, 128) == 16);     // 4 windows of 16 rows: 1 tile each
-  CHECK(jf::attn_units_estimate(128, 4, 44, 4, 7, 128) == 32);    // 4 windows of 32 rows: 2 tiles each
-  CHECK(jf::attn_units_estimate(512, 4, 132, 4, 7, 128) == 112);  // 4 windows of 128 rows: 7 tiles each
-  CHECK(jf::attn_units_estimate(512, 4, 100, 4, 7, 128) == 100);  // capped by the launch bound
+  // unit estimates: rows spread over the chains, whole tiles per chain and KV head
+  CHECK(jf::attn_units_estimate(32, 1, 12, 4, 7, 126) == 8);      // 224 query rows: 2 tiles x 4 heads
+  CHECK(jf::attn_units_estimate(64, 4, 32, 4, 7, 126) == 16);     // 4 windows of 16 rows: 1 tile each
+  CHECK(jf::attn_units_estimate(128, 4, 44, 4, 7, 126) == 32);    // 4 windows of 32 rows: 2 tiles each
+  CHECK(jf::attn_units_estimate(512, 4, 132, 4, 7, 126) == 128);  // 4 windows of 128 rows: 8 tiles each
+  CHECK(jf::attn_units_estimate(512, 4, 100, 4, 7, 126) == 100);  // capped by the launch bound
   CHECK(jf::attn_units_estimate(5, 0, 8, 2, 4, 128) == 2);        // no chain count: one chain
-  // waves: clustered ceil(u / 15), unclustered ceil(8 u / 152); ties to the clustered form
-  CHECK(jf::attn_use_clusters(15, 8, 15, 152));                    // 1 wave either way
-  CHECK(!jf::attn_use_clusters(16, 8, 15, 152));                   // 2 waves against 1
-  CHECK(jf::attn_use_clusters(28, 8, 15, 152));                    // 2 against 2
-  CHECK(!jf::attn_use_clusters(112, 8, 15, 152));                  // 8 against 6
-  CHECK(jf::attn_use_clusters(3, 8, 0, 152) == jf::attn_use_clusters(3, 8, 1, 152));  // no count: 1
-  // the sweep's points (7B shape): the form the rule picks is the one measured faster
-  CHECK(clustered(32, 1, 4, 7));      // decode, 32 rows
-  CHECK(!clustered(64, 1, 4, 7));     // 64-row window: 3.96 (clustered) against 3.73 ms
-  CHECK(clustered(128, 1, 4, 7));     // 128-row window: the clustered fold 5% faster at equal waves
-  CHECK(clustered(192, 1, 4, 7));     // 192 rows: 5.55 against 5.70 ms
-  CHECK(!clustered(64, 4, 4, 7));     // B = 4, n = 16: at 32k 8.83 against 6.07 ms
-  CHECK(!clustered(128, 4, 4, 7));    // B = 4, n = 32
-  CHECK(!clustered(512, 4, 4, 7));    // B = 4, n = 128: at 32k 29.21 against 24.44 ms
-  CHECK(!clustered(384, 1, 4, 7));    // the knee's 384 rows: 9.75 against 9.20 ms
-  // the small model (2 KV heads, 4 query heads each): a 256-row window is unclustered, one row is not
-  CHECK(!clustered(256, 1, 2, 4));
-  CHECK(clustered(1, 1, 2, 4));
+  // no residency known: one cluster at a time
+  const int none[4] = {0, 0, 0, 0};
+  CHECK(jf::attn_ctas_per_unit(3, none) == 8);
+  // the 7B shape: one wave of the widest clusters that fit
+  CHECK(ctas(32, 1, 4, 7) == 8);    // 8 units
+  CHECK(ctas(64, 1, 4, 7) == 4);    // 16
+  CHECK(ctas(128, 1, 4, 7) == 4);   // 32
+  CHECK(ctas(192, 1, 4, 7) == 2);   // 44
+  CHECK(ctas(384, 1, 4, 7) == 1);   // 88
+  CHECK(ctas(512, 1, 4, 7) == 1);   // 116
+  CHECK(ctas(64, 4, 4, 7) == 4);    // four sequences: 16
+  CHECK(ctas(128, 4, 4, 7) == 4);   // 32
+  CHECK(ctas(512, 4, 4, 7) == 1);   // 128
+  // the small model: 16 units of a 256-row window on clusters of 4, one row on clusters of 8; prefills of 64,
+  // 300, 700 and 1,300 rows
+  CHECK(ctas(256, 1, 2, 4) == 4);
+  CHECK(ctas(1, 1, 2, 4) == 8);
+  CHECK(ctas(64, 1, 2, 4) == 8);
+  CHECK(ctas(300, 1, 2, 4) == 4);
+  CHECK(ctas(700, 1, 2, 4) == 2);
+  CHECK(ctas(1300, 1, 2, 4) == 1);
   std::printf("ok\n");
   return 0;
 }

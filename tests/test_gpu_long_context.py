@@ -9,7 +9,7 @@ partial states. Checked here:
   (a row's arithmetic does not depend on the rows in flight with it);
 * greedy Jacobi decoding equals greedy AR decoding on the device at 2540 committed tokens
   (small model) and at 16384 committed tokens (1.5B shape), and with a 256-row window whose
-  attention runs the unclustered form of the kernel.
+  attention runs on narrower clusters than one row's.
 """
 import numpy as np
 import pytest
@@ -99,12 +99,11 @@ def test_jacobi_equals_ar_16k_context_1p5b():
         ctx.close()
 
 
-def test_unclustered_attention_decodes_like_clustered():
+def test_narrow_clusters_decode_like_wide_ones():
     """A 256-row Jacobi window on the small model has 16 attention units (2 KV heads x 8 query
-    tiles), more than the 15 8-CTA clusters of the attention kernel that a GB300 holds at once: as
-    clusters they take two waves, as independent CTAs (128) one, so its forwards run the unclustered
-    form (the last lane of a unit folds all its rows). AR forwards (one row, two units) run the
-    clustered form. Both fold in lane order with the same arithmetic: the tokens are identical."""
+    tiles), more than the 15 8-CTA clusters of the attention kernel that a GB300 holds at once, so its
+    forwards run on clusters of 4, each CTA walking two key lanes. AR forwards (one row, two units) run
+    on clusters of 8. Both fold in lane order with the same arithmetic: the tokens are identical."""
     need_gpu()
     from paper_2512_14681_gb300.jacobi import Context, Gen
 
