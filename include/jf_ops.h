@@ -27,10 +27,11 @@ jf_status jf_op_gemm_workspace_bytes(int N, int K, int M, int k_splits, size_t* 
  * every projection of the forward pass.
  * dtype JF_BF16: W [N][K] and X [M][K] bf16 (device, 16-byte aligned, K % 8 == 0), tcgen05
  *   tensor cores fed by TMA; JF_F32: W, X fp32, CUDA cores.
- * Y: device fp32 [M][N]. workspace: device, jf_op_gemm_workspace_bytes() bytes, in any state: each
- * call clears the tickets it uses, so calls of different shapes may share one on a stream (bf16 only;
- * they are zero again after the call). err_word: device int that receives a device error code (0 =
- * none); the caller reads it after synchronising. */
+ * Y: device fp32 [M][N]. workspace: device, jf_op_gemm_workspace_bytes() bytes, zero-filled before
+ * its first use and after a call that left an error code. Calls of different shapes may then share it
+ * on a stream: tickets are zero again after a call, and partial tiles that a call of another shape left
+ * where this one's tickets are count as zero. err_word: device int that receives a device error code
+ * (0 = none); the caller reads it after synchronising. */
 jf_status jf_op_gemm(int dtype, const void* W, const void* X, float* Y, int N, int K, int M, int k_splits,
                      void* workspace, size_t workspace_bytes, int* err_word, void* cuda_stream);
 

@@ -302,6 +302,12 @@ JF_DEV void epilogue_chunk(const GemmEpi& e, const float (&v)[16], const EpiThre
   }
 }
 
+// A split tile's CTAs draw tickets with atomicDec, which starts anew from 0 and from any word above the split
+// count. jf_op_gemm's tickets lie behind its partial tiles, at a place that depends on the shape, and another
+// shape's call on the same workspace may have left partials there: they are stored complemented, so that none
+// of them reads as 1 .. 7 (the complements of those are NaNs that no sum gives: a sum's NaN is 0x7fffffff).
+JF_DEV float complement(float v) { return __uint_as_float(~__float_as_uint(v)); }
+
 // Shared tail of both mainloops, run by the epilogue threads: the partial tile for EPI_PARTIAL;
 // otherwise ticketing for split-K, then the epilogue. get(c0, v) fills this thread's 16 accumulator
 // values of columns c0..c0+15. am: this CTA's argmax entries.
@@ -313,17 +319,17 @@ JF_DEV void finish_tile(const GemmParams& p, Get get, float* xs, int* sflag, int
   int ncols = p.M - m0;
   if (ncols > BN) ncols = BN;
   const int nchunks = (ncols + 15) >> 4;
-  auto store_partial = [&]() {
+  auto store_partial = [&](auto word) {
     float* mine = p.ws + ((size_t)tile_lin * p.k_splits + split) * (size_t)BN * kTileN;
     for (int c = th.half; c < nchunks; c += NH) {
       float v[16];
       get(c * 16, v);
 #pragma unroll
-      for (int j = 0; j < 16; ++j) mine[(c * 16 + j) * kTileN + th.row] = v[j];
+      for (int j = 0; j < 16; ++j) mine[(c * 16 + j) * kTileN + th.row] = word(v[j]);
     }
   };
   if constexpr (EPI == EPI_PARTIAL) {
-    store_partial();
+    store_partial([](float v) { return v; });
   } else if (p.k_splits == 1) {
     for (int c = th.half; c < nchunks; c += NH) {
       float v[16];
@@ -331,12 +337,12 @@ JF_DEV void finish_tile(const GemmParams& p, Get get, float* xs, int* sflag, int
       epilogue_chunk<T, EPI>(p.epi, v, th, n0, m0, c * 16, xs, n_tile, am);
     }
   } else {
-    store_partial();
+    store_partial(complement);
     __threadfence();
     th.sync_all();
     if (th.first()) {
-      const int t = atomicAdd(p.tile_counter + tile_lin, 1);
-      *sflag = (t == p.k_splits - 1);
+      // 0 or a stale word -> k_splits - 1 -> ... -> 1 -> 0
+      *sflag = atomicDec(reinterpret_cast<unsigned*>(p.tile_counter) + tile_lin, (unsigned)p.k_splits - 1u) == 1u;
     }
     th.sync_all();
     const bool last = *sflag != 0;
@@ -357,7 +363,7 @@ JF_DEV void finish_tile(const GemmParams& p, Get get, float* xs, int* sflag, int
           const float* src = base + (size_t)(s0 + s) * BN * kTileN;
 #pragma unroll
           for (int j = 0; j < 16; ++j)
-            part[s][j] = (s0 + s < p.k_splits) ? __ldcg(src + (c * 16 + j) * kTileN + th.row) : 0.0f;
+            part[s][j] = (s0 + s < p.k_splits) ? complement(__ldcg(src + (c * 16 + j) * kTileN + th.row)) : 0.0f;
         }
 #pragma unroll
         for (int s = 0; s < 4; ++s) {
@@ -369,7 +375,6 @@ JF_DEV void finish_tile(const GemmParams& p, Get get, float* xs, int* sflag, int
       }
       epilogue_chunk<T, EPI>(p.epi, v, th, n0, m0, c * 16, xs, n_tile, am);
     }
-    if (th.first()) p.tile_counter[tile_lin] = 0;
   }
 }
 

@@ -106,7 +106,7 @@ struct GemmParams {
   int n_tiles, m_tiles, k_splits, kb_total;
   int grid;            // persistent CTAs (bf16 path): at most one per SM
   float* ws;           // split-K partials [n_tiles][m_tiles][k_splits][BN][128]
-  int* tile_counter;   // [m_tiles*n_tiles], zero between launches
+  int* tile_counter;   // [m_tiles*n_tiles] tickets: zero, or stale partials, before a launch; zero after it
   int* err;
   unsigned long long wait_ns;  // limit of each bounded wait
   // bf16 path: programmatic launch. Only where W was complete before the kernels that may still run began (a

@@ -1661,8 +1661,6 @@ jf_status jf_op_gemm(int dtype, const void* W, const void* X, float* Y, int N, i
     if (gemm_prepare() != cudaSuccess) return JF_ECUDA;  // once per device
     CUtensorMap tA, tB;
     if (!make_tmap(&tA, W, K, N, kTileN) || !make_tmap(&tB, X, K, M, gemm_box_rows(bn, M))) return JF_ECUDA;
-    // the tickets lie behind the partial tiles: another shape's call may have left its partials there
-    if (cudaMemsetAsync(p.tile_counter, 0, rup((size_t)nt * mt * 4, 256), st) != cudaSuccess) return JF_ECUDA;
     e = launch_gemm_bf16(tA, tB, p, bn, st);
   } else {
     if (gemm_prepare() != cudaSuccess) return JF_ECUDA;

@@ -270,7 +270,7 @@ def op_gemm(W, X, k_splits: int = 0, stream=None):
     dtype = J.JF_BF16 if W.dtype == torch.bfloat16 else J.JF_F32
     nb = C.c_size_t()
     _check(lib, None, lib.jf_op_gemm_workspace_bytes(N, K, M, k_splits, C.byref(nb)))
-    ws = torch.empty(max(nb.value, 16), dtype=torch.uint8, device=W.device)
+    ws = torch.zeros(max(nb.value, 16), dtype=torch.uint8, device=W.device)
     err = torch.zeros(1, dtype=torch.int32, device=W.device)
     Y = torch.empty((M, N), dtype=torch.float32, device=W.device)
     s = stream if stream is not None else torch.cuda.current_stream()

@@ -98,9 +98,11 @@ def test_gemm_f32_matches_oracle():
 
 
 @pytest.mark.parametrize("first,second", [((300, 4), (32, 4)), ((32, 4), (300, 4)), ((200, 8), (64, 2)), ((600, 2), (600, 3))])
-def test_gemm_bf16_shapes_share_a_workspace(first, second):
+@pytest.mark.parametrize("tiny", [False, True])
+def test_gemm_bf16_shapes_share_a_workspace(first, second, tiny):
     """Calls of two shapes through one workspace zeroed once: the tickets of the second one lie where the
-    first one's partial tiles may be. Every element of Y is written, with the bits of a call of its own."""
+    first one's partial tiles may be (tiny: partial sums of 2^-149, whose bits are a small integer's). Every
+    element of Y is written, with the bits of a call of its own."""
     torch = need_gpu()
     import ctypes
 
@@ -108,15 +110,19 @@ def test_gemm_bf16_shapes_share_a_workspace(first, second):
     from paper_2512_14681_gb300.jacobi import op_gemm
 
     lib, N, K = J.load(), 640, 2048
-    W = _bf16(torch, I.random_array((N, K), seed=21, scale=0.5))
     nb = ctypes.c_size_t()
     need = 0
     for M, splits in (first, second):
         assert lib.jf_op_gemm_workspace_bytes(N, K, M, splits, ctypes.byref(nb)) == J.JF_OK
         need = max(need, nb.value)
     ws, err = torch.zeros(need, dtype=torch.uint8, device="cuda"), torch.zeros(1, dtype=torch.int32, device="cuda")
-    for M, splits in (first, second):
+    for k, (M, splits) in enumerate((first, second)):
+        W = _bf16(torch, I.random_array((N, K), seed=21, scale=0.5))
         X = _bf16(torch, I.random_array((M, K), seed=M, scale=0.5))
+        if tiny and k == 0:
+            W.fill_(2.0**-75)
+            X.zero_()
+            X[:, ::256] = 2.0**-74  # one product in each split
         Y = torch.full((M, N), float("nan"), device="cuda")
         assert lib.jf_op_gemm(J.JF_BF16, W.data_ptr(), X.data_ptr(), Y.data_ptr(), N, K, M, splits, ws.data_ptr(), need,
                               err.data_ptr(), torch.cuda.current_stream().cuda_stream) == J.JF_OK
