@@ -109,9 +109,9 @@ struct GemmParams {
   int* tile_counter;   // [m_tiles*n_tiles] tickets: zero, or stale partials, before a launch; zero after it
   int* err;
   unsigned long long wait_ns;  // limit of each bounded wait
-  // bf16 path: programmatic launch. Only where W was complete before the kernels that may still run began (a
-  // context's weights): its first tiles are requested ahead of the dependency wait.
-  bool overlap;
+  // bf16 path: W was complete before any kernel that may still run began (a context's weights), so that its first
+  // tiles may be requested ahead of the dependency wait
+  bool w_ready;
   GemmEpi epi;
 };
 

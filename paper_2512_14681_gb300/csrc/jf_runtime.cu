@@ -490,7 +490,7 @@ cudaError_t gemm(jf_ctx* c, const CUtensorMap& tmA, const void* W, const void* X
   p.err = c->err;
   p.wait_ns = c->wait_ns;
   p.grid = c->num_sms;
-  p.overlap = true;
+  p.w_ready = true;
   p.epi = epi;
   p.epi.M = M;
   p.epi.N = N;
