@@ -385,11 +385,13 @@ void free_pinned(jf_ctx* c) {
   if (c->words_out) cudaFreeHost(c->words_out);
 }
 
-// The error word that the stream's work left, read with it (the stream is idle); a set one is cleared.
+// The error word that the stream's work left, read with it (the stream is idle); a set one is cleared, and so
+// are the split-K tickets: a projection whose waits gave up has not drawn all of its own.
 jf_status take_err(jf_ctx* c, int e) {
   if (e) {
     int z = 0;
     cudaMemcpyAsync(c->err, &z, 4, cudaMemcpyHostToDevice, c->st);
+    cudaMemsetAsync(c->gemm_counter, 0, c->O.am_v1 - c->O.gemm_counter, c->st);
     cudaStreamSynchronize(c->st);
   }
   return check_err_word(c, e);
