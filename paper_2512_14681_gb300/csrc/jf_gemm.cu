@@ -686,6 +686,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
       const int n_tile = w.n_tile * kCtas + rank;
       if (n_tile < p.n_tiles)  // (the last pair's second tile may not exist)
         finish_tile<bf16, BN, EPI>(p, get, xs, sflag, n_tile, w.split, w.m_tile, th, am);
+      if (u + unit_step >= total_units) break;  // nobody waits for the last accumulator to be free
       tc_fence_before();
       th.sync_all();
       if (tid == 0) {
