@@ -72,9 +72,9 @@ DEFAULT_WORKLOAD = next(iter(WORKLOADS))
 ALIASES = {"7b": DEFAULT_WORKLOAD, "7b-p0.1": list(WORKLOADS)[1], "7b-p0.7": list(WORKLOADS)[2],
            "1.5b": list(WORKLOADS)[3], "7b-mb4-rr": list(WORKLOADS)[4], "7b-mr-k2n64": list(WORKLOADS)[5]}
 # DRAM bytes (read + write) per launch of the gate/up projection at M = 32 rows: dram__bytes_read.sum
-# + dram__bytes_write.sum, mean of two captured launches of the current kernel (271.87 MB weights and
-# activations read, 0.5 and 3.0 MB SwiGLU output written). Set to None whenever the kernel changes.
-GATEUP_TRAFFIC_BYTES = 273_629_824
+# + dram__bytes_write.sum, mean of four captured launches of the current kernel (271.86 MB weights and
+# activations read, 0.5 to 3.2 MB SwiGLU output written). Set to None whenever the kernel changes.
+GATEUP_TRAFFIC_BYTES = 273_074_240
 
 
 def _peaks():

@@ -309,12 +309,13 @@ JF_DEV void fold_row_block(const AttnParams& a, const AttnUnit& u, int ui, int r
 // 128 / n_ctas of the rows. Every form computes the same lane states and folds them in lane order,
 // so their results are bit-identical.
 //
-// What bounds it: a 128-key chunk takes about 2000 cycles of a CTA, of which the softmax warps compute
-// 1500 (row maxima, 64 exponentials a thread, P) and the tensor cores about 1100. With every warp
+// What bounds it: a 128-key chunk takes about 2000 cycles of a CTA (ncu, 32,768 keys: the tensor pipe is busy
+// for 1020 of them, ex2 and the issue slots for 21% and 41%), the chain of the softmax warps (scores out of
+// tensor memory, the row maxima's barrier, 64 exponentials a thread, P back). With every warp
 // loading K/V by cp.async, waiting for each MMA and adding P V in registers a chunk took 4900 (30% of
 // it the copies' issue). One 7B layer at P = 32768: 32 rows 204 -> 147 us, 128 rows 330 -> 198 us; 512
 // rows at 4096: 398 -> 309 us. Long units are bound by the chunk step. At decode sizes (P = 1024, 32
-// rows: 9.2 -> 8.9 us of attention a layer) the prologue and the fold dominate: lane states pass through
+// rows: 9.2 us of attention a layer, as before) the prologue and the fold dominate: lane states pass through
 // L2 in 16-byte pieces ([dim / 4][row][4]; one value a store took 1 us more), and the code is kept small
 // (unrolled loaders made a first pass over a layer 4 us slower).
 template <bool kWhole>

@@ -680,8 +680,8 @@ cudaLaunchConfig_t pdl_cfg(dim3 grid, dim3 block, size_t smem, cudaStream_t st, 
 // Host/device hand-over of a call, a few KB: latency bounds it, so every array goes in one launch (a
 // forward took four copies from pageable memory and a synchronisation before its first kernel, and two
 // copies, each waited for, after its last). One layer of the 7B shape, 32 rows over 1,024 tokens: 181 ->
-// 150 us a call; of the 1.5B shape, 19 rows over 777: 118 -> 88; a 4,000-token prefill through one 7B layer
-// 2,213 -> 2,054. Neither triggers its dependents, and the forward's first kernel (k_embed) is launched without
+// 153 us a call; of the 1.5B shape, 19 rows over 777: 118 -> 90; a 4,000-token prefill through one 7B layer
+// 2,213 -> 2,050. Neither triggers its dependents, and the forward's first kernel (k_embed) is launched without
 // the programmatic attribute, so that it starts after these writes are complete and visible.
 __global__ void __launch_bounds__(256) k_copy_words(const WordCopies w) {
   for (int c = 0; c < w.n_copies; ++c)

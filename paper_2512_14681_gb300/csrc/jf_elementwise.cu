@@ -66,8 +66,8 @@ __global__ void k_rope_table(float2* tab, int n_pos, int half, double theta) {
 // programmatic attribute: it starts once everything before it on the stream is complete and visible, and the
 // forward's other kernels start after it. They may therefore read what was written before the forward (rows,
 // positions, the chain table, pages, weights) ahead of their own dependency wait; that wait alone would not
-// order such a read, as each kernel lets the next one in at its entry. The boundary costs nothing that was
-// hidden: what precedes a forward is a hand-over kernel of a few KB or another graph launch.
+// order such a read, as each kernel lets the next one in at its entry. What precedes it is another graph
+// launch, where the boundary costs nothing, or a hand-over kernel (2 us of a call).
 template <typename T>
 __global__ void k_embed(const T* __restrict__ E, const int* __restrict__ tok, float* __restrict__ x, int d, int V,
                         int* err) {

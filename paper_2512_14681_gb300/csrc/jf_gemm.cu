@@ -406,7 +406,8 @@ JF_DEV Unit unit_of(const GemmParams& p, int u) {
 // stage instead of 48), rank 0 issues the MMAs of both, and each drains its own 128 rows. With
 // one CTA per tile the operands, not the tensor cores, bounded it: 48 KB a 512-cycle stage is more than
 // an SM draws from L2, and only four such stages fit. gate/up (37888 x 3584) at 512 rows: 110.6 ->
-// 104.9 us a call (1.33 PFLOP/s); prefill of 4,000 tokens through one 7B layer 2.39 -> 2.29 ms.
+// 104.9 us a call, the launch 103.5 -> 87 (ncu; 1.6 PFLOP/s, tensor pipe 77% of the active cycles); prefill of
+// 4,000 tokens through one 7B layer 2.39 -> 2.29 ms.
 // ---------------------------------------------------------------------------------------------
 constexpr int EPI_HALVES = 2, PRODUCER_WARP = 4 * EPI_HALVES, MMA_WARP = PRODUCER_WARP + 1;
 constexpr int TC_THREADS = 32 * (MMA_WARP + 1);
@@ -724,8 +725,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
 // the CTAs of the cluster in rank order (read from their shared memory), are added in a fixed order that
 // depends on N and K alone. These models' matrices are small (a 256 x 1024 one is two feature tiles), so
 // latency bounds the kernel: it is spread over 8-152 SMs instead of one CTA per tile whose threads each
-// walked a weight row (a jf_op_gemm call of 4096 x 1024, 40 rows: 158 -> 41 us, most of which is now the
-// call itself; the tiny fp32 decoder's generation, with the fp32 attention: 35.9 -> 6.2 ms).
+// walked a weight row (a jf_op_gemm call of 4096 x 1024, 40 rows: 150 -> 53 us, of which a launch takes 26-35;
+// the tiny fp32 decoder's generation, with the fp32 attention: 33.0 -> 5.3 ms).
 // ---------------------------------------------------------------------------------------------
 constexpr int F32_BK = 32;
 constexpr int F32_STAGES = 4;
