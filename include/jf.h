@@ -141,7 +141,9 @@ jf_status jf_jacobi_step(jf_ctx* ctx, int seq, int n_blocks, const jf_block* blo
 
 /* Forward of `n_rows` tokens (host) of sequence `seq` at positions P .. P+n_rows-1 with a causal
  * mask, WITHOUT committing: fp32 logits [n_rows][V], final residual stream [n_rows][d] (before
- * the final norm) and argmax [n_rows], each optional (host). n_rows <= logits_rows. */
+ * the final norm) and argmax [n_rows], each optional (host). n_rows <= logits_rows.
+ * A row whose logits are all NaN has no greedy token: here, in a step's predictions and in jf_prefill's
+ * next_token it reads 0x7fffffff, and a generation ends with JF_EDEVICE. */
 jf_status jf_forward_logits(jf_ctx* ctx, int seq, int n_rows, const int32_t* tokens, float* logits, float* hidden,
                             int32_t* argmax);
 

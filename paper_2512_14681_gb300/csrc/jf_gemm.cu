@@ -62,7 +62,8 @@ JF_DEV uint8_t* align1024(uint8_t* p) {
 // ---------------------------------------------------------------------------------------------
 // Greedy argmax. Logits are compared through keys that preserve their order as unsigned integers (-0
 // counts as +0, NaN as the lowest, key 0). A row without a number gets the index kAmNoIndex, which no
-// vocabulary holds: the callers see it, and the next forward's embedding reports it. Every CTA keeps a running entry (best key, its lowest index,
+// vocabulary holds: the callers see it, and the next forward's embedding reports it. Every CTA keeps a
+// running entry (best key, its lowest index,
 // runner-up key) of every row over the vocabulary tiles it takes: in shared memory for up to
 // kAmTableRows rows, otherwise in its global slot; k_argmax_finish merges the CTAs' slots. The merge is
 // associative and commutative, so the result does not depend on which CTA took which tile. With
@@ -602,7 +603,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
       for (int u = first_unit; u < total_units && ok; u += unit_step, ++i) {
         const Unit w = unit_of(p, u);
         const int acc = i & 1;
-        if (i >= 2 && !__all_sync(0xffffffffu, mbar_wait_bounded(tempty0 + 8 * acc, (uint32_t)((i >> 1) - 1) & 1u, p.wait_ns))) {
+        const uint32_t prev = (uint32_t)((i >> 1) - 1) & 1u;  // phase of the accumulator's previous use
+        if (i >= 2 && !__all_sync(0xffffffffu, mbar_wait_bounded(tempty0 + 8 * acc, prev, p.wait_ns))) {
           if (lane == 0) jf_set_error(p.err, JF_DERR_TIMEOUT_EPI);
           break;
         }
